@@ -26,6 +26,7 @@
 #include "vspec_kernels_coltc.cuh"
 #include "vspec_kernels_tcfir.cuh"
 #include "vspec_ring.cuh"
+#include "vspec_row2048.cuh"
 #include "vspec_bp.cuh"
 #include "vspec_internal.h"
 
@@ -177,6 +178,9 @@ struct vspec_plan {
     bool kahan = false;        // compensated accumulation at every level
     void *partial_comp = nullptr, *out_comp = nullptr;
     int *tc_status = nullptr;  // bounded-wait flag of the tensor-core or ring kernel
+    int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel (in twB's allocation)
+    float2 *twBt = nullptr;      // its twiddles (in twB's allocation)
+    bool row_groups = false;     // kernel B is row2048_group_kernel
     // persistent ring form (VSPEC_PLAN_RING): Z holds ringR slots of ringS
     // spectra, `partial` ring_sets partial-sum sets
     bool ring = false;
@@ -859,16 +863,19 @@ vspec_status build_plan(vspec_plan *p) {
         p->passB[1].r == 16 && p->passB[2].r == 8) {
         using namespace vspec;
         const bool k = p->kahan, f = p->fir_b;
-        if (p->npol == 2 && coltc)  // scratch elements in the tensor-core column kernel's order
-            p->kernelB = k ? (const void *)row2048_kernel<2, true, false, true> : (const void *)row2048_kernel<2, false, false, true>;
+        p->row_groups = p->npol == 2 && !k && !f;
+        if (p->row_groups)  // coltc: scratch elements in the tensor-core column kernel's order
+            p->kernelB = coltc ? (const void *)row2048_group_kernel<true> : (const void *)row2048_group_kernel<false>;
+        else if (p->npol == 2 && coltc)
+            p->kernelB = (const void *)row2048_kernel<2, true, false, true>;
         else if (p->npol == 2)
             p->kernelB = k ? (f ? (const void *)row2048_kernel<2, true, true> : (const void *)row2048_kernel<2, true, false>)
-                           : (f ? (const void *)row2048_kernel<2, false, true> : (const void *)row2048_kernel<2, false, false>);
+                           : (const void *)row2048_kernel<2, false, true>;
         else
             p->kernelB = k ? (f ? (const void *)row2048_kernel<1, true, true> : (const void *)row2048_kernel<1, true, false>)
                            : (f ? (const void *)row2048_kernel<1, false, true> : (const void *)row2048_kernel<1, false, false>);
-        p->TB = 256;
-        p->smemB = 2 * (size_t)kRow2048Stride * elem;
+        p->TB = p->row_groups ? Row2048::THREADS : 256;
+        p->smemB = p->row_groups ? Row2048::smem : 2 * (size_t)kRow2048Stride * elem;
         p->formB = "row2048";
         p->fold2048 = N2 >= 16 && !p->kahan;
     }
@@ -931,7 +938,14 @@ vspec_status build_plan(vspec_plan *p) {
     const int Lc = (pfb ? p->P : 1) * N;
     if ((st = dev_alloc((void **)&p->coef, sizeof(float) * (size_t)Lc, &tot))) return st;
     if ((st = dev_alloc((void **)&p->twA, sizeof(float2) * (size_t)std::max(1, twA_n), &tot))) return st;
-    if ((st = dev_alloc((void **)&p->twB, sizeof(float2) * (size_t)std::max(1, twB_n), &tot))) return st;
+    // with the row kernel's own twiddle order and wait flag after the table
+    const int twBt_n = p->row_groups ? vspec::Row2048::TW1 + vspec::Row2048::TW2 : 0;
+    if ((st = dev_alloc((void **)&p->twB, sizeof(float2) * (size_t)(std::max(1, twB_n) + twBt_n + 1), &tot))) return st;
+    if (p->row_groups) {
+        p->twBt = p->twB + twB_n;
+        p->row_status = reinterpret_cast<int *>(p->twBt + twBt_n);
+        VSPEC_CUDA(cudaMemset(p->row_status, 0, sizeof(int)));
+    }
     if ((st = dev_alloc((void **)&p->twZ, sizeof(float2) * (size_t)N, &tot))) return st;
     if ((st = dev_alloc((void **)&p->invA, sizeof(int) * (size_t)N2, &tot))) return st;
     if ((st = dev_alloc((void **)&p->invB, sizeof(int) * (size_t)N1, &tot))) return st;
@@ -984,6 +998,10 @@ vspec_status build_plan(vspec_plan *p) {
         for (const Pass &ps : p->passB)
             if (ps.m * (ps.r - 1) > 0)
                 vspec::gen_pass_tw_kernel<<<(ps.m * (ps.r - 1) + 255) / 256, 256, 0, s0>>>(p->twB, ps);
+        if (p->row_groups) {
+            vspec::gen_pass_tw_t_kernel<<<(vspec::Row2048::TW1 + 255) / 256, 256, 0, s0>>>(p->twBt, p->passB[0]);
+            vspec::gen_pass_tw_t_kernel<<<1, 256, 0, s0>>>(p->twBt + vspec::Row2048::TW1, p->passB[1]);
+        }
         vspec::gen_twz_kernel<<<(N + 255) / 256, 256, 0, s0>>>(p->twZ, N, N1, N2, d_kA);
         if (p->tc_cols && !p->tc_int8) {
             vspec::gen_coltc_operand_kernel<<<(4 * N2 * N2 + 255) / 256, 256, 0, s0>>>(p->dftop, N2);
@@ -1591,6 +1609,8 @@ static void make_params(const vspec_plan *p, const int8_t *d_in, int nspectra, v
     cb.partial = p->partial;
     cb.partial_comp = p->partial_comp;
     cb.twB = p->twB;
+    cb.twBt = p->twBt;
+    cb.wait_status = p->row_status;
     cb.N = p->N;
     cb.N1 = p->N1;
     cb.N2 = p->N2;
@@ -2004,12 +2024,17 @@ vspec_status vspec_plan_set_host_mode(vspec_plan *plan, int mode, size_t chunk_b
 
 vspec_status vspec_plan_check(vspec_plan *plan) {
     if (!plan) return VSPEC_ERR_INVALID_ARG;
-    if (!plan->tc_status) return VSPEC_OK;
-    int h = 0;
-    VSPEC_CUDA(cudaMemcpy(&h, plan->tc_status, sizeof(int), cudaMemcpyDeviceToHost));
-    if (!h) return VSPEC_OK;
-    VSPEC_CUDA(cudaMemset(plan->tc_status, 0, sizeof(int)));
-    g_last_error = "a bounded wait for the tensor cores expired";
+    bool expired = false;
+    for (int *word : {plan->tc_status, plan->row_status, plan->assist ? plan->assist->row_status : nullptr}) {
+        if (!word) continue;
+        int h = 0;
+        VSPEC_CUDA(cudaMemcpy(&h, word, sizeof(int), cudaMemcpyDeviceToHost));
+        if (!h) continue;
+        VSPEC_CUDA(cudaMemset(word, 0, sizeof(int)));
+        expired = true;
+    }
+    if (!expired) return VSPEC_OK;
+    g_last_error = "a bounded wait for the tensor cores or for a row's copy expired";
     return VSPEC_ERR_DEVICE_TIMEOUT;
 }
 

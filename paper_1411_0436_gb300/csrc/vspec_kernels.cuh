@@ -98,6 +98,8 @@ struct RowParams {
     void *partial;       // [group][pos][posB] of Elem::Acc, accumulated into
     void *partial_comp;  // Kahan compensation of `partial` (compensated plans only)
     const float2 *twB;   // per-pass twiddles of the length-N1 row DFTs
+    const float2 *twBt;  // 2048-point rows: passes 1 and 2 in [q - 1][j] order (row2048_group_kernel)
+    int *wait_status;    // set to 1 if a bounded wait for a row's copy gave up (row2048_group_kernel)
     int N, N1, N2, RB, npass;
     int lN1, lRB;        // log2 N1, log2 RB
     Pass pass[kMaxPasses];
@@ -1229,6 +1231,9 @@ __global__ void __launch_bounds__(256, 2) rowfft_detect_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------ kernel B, 2048 --
+// Single-polarisation, compensated and one-row plans, and the row bodies of
+// the persistent forms; other dual-pol plans run row2048_group_kernel
+// (vspec_row2048.cuh).
 // Rows of 2048 points (RB = 1; passes radix 16, 16, 8), two spectra at a
 // time. In the radix-16 passes (128 butterflies each) the block's halves
 // transform one spectrum each, synchronising on their own named barrier;
