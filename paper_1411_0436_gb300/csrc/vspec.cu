@@ -140,6 +140,7 @@ struct vspec_plan {
     const char *formA = "general";   // kernel A's form (vspec_plan_describe)
     const char *formB = "general";   // kernel B's form
     int num_sms = 0, occA = 1, occB = 1;
+    int maxB = 1;                    // kernel-B CTAs per SM that tuning limits and partial-sum slots allow for
     int sc_max = 1;                  // spectra per chunk
     int sc_cap = 1, slots_cap = 1;   // largest chunk a tuning may ask for; slots allocated
     int sc_alloc = 1;                // chunk spectra the scratch holds now
@@ -930,7 +931,9 @@ vspec_status build_plan(vspec_plan *p) {
     p->sc_max = std::min({p->sc_cap, kMaxChunkSpectra, (int)std::max<size_t>(1, kScratchBudget / per_spec)});
     if (p->fir_b) p->sc_cap = p->sc_max = kMaxChunkSpectra;  // launch length only: no scratch
     // partial-sum slots for the largest kernel-B launch a tuning may ask for
-    p->slots_cap = slots_for(p, kMaxWaves * p->num_sms * p->occB);
+    // (row2048_group_kernel runs one CTA per SM, but keeps the limits of two)
+    p->maxB = p->row_groups ? std::max(2, p->occB) : p->occB;
+    p->slots_cap = slots_for(p, kMaxWaves * p->num_sms * p->maxB);
 
     // device tables and scratch
     vspec_status st;
@@ -1242,7 +1245,7 @@ vspec_status vspec_plan_get_tuning(const vspec_plan *plan, vspec_tuning *current
         cur.blocks_b = tk->blocks_b;
         lim.chunk_spectra = tk->sc_cap;
         lim.blocks_a = kMaxWaves * tk->num_sms * tk->occA;
-        lim.blocks_b = kMaxWaves * tk->num_sms * tk->occB;
+        lim.blocks_b = kMaxWaves * tk->num_sms * tk->maxB;
     }
     if (plan->fused) {
         const bool can_assist = plan->assist && plan->num_sms - plan->cluster * plan->nclusters >= kAssistMinSms;
