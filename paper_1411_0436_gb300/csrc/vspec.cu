@@ -394,22 +394,22 @@ vspec_status launch(vspec_plan *p, int kind, int spectra, const void *fn, dim3 g
 }
 
 // Fold `slots` partial-sum slots of p->partial (and p->partial_comp in
-// compensated plans) into d_accum: with more than 128 slots, first sum each
+// compensated plans; slots of nsub bands in sub-band calls) into d_accum: with more than 128 slots, first sum each
 // group of 16 slots into its first slot, then fold the group sums.
-vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, cudaStream_t st) {
-    int groups = slots, stride = 1;
+vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, cudaStream_t st, int nsub = 1) {
+    int groups = slots, stride = nsub;  // a slot holds the nsub bands one after another
     const int N = p->N, N1 = p->N1, N2 = p->N2;
     if (slots > 128) {
         groups = (slots + 15) / 16;
-        stride = 16;
+        stride = 16 * nsub;
         const void *fold = p->npol == 2 ? (p->kahan ? (const void *)vspec::fold_slots_kernel<2, true>
                                                     : (const void *)vspec::fold_slots_kernel<2, false>)
                                         : (p->kahan ? (const void *)vspec::fold_slots_kernel<1, true>
                                                     : (const void *)vspec::fold_slots_kernel<1, false>);
         void *part = p->partial, *pcomp = p->partial_comp;
-        int ns = slots, n = N;
+        int ns = slots, n = N * nsub;
         void *argsF[] = {&part, &pcomp, &ns, &n};
-        vspec_status r = launch(p, 2, 0, fold, dim3((N + 31) / 32, groups), dim3(32, 8), argsF, 0, st);
+        vspec_status r = launch(p, 2, 0, fold, dim3((n + 31) / 32, groups), dim3(32, 8), argsF, 0, st);
         if (r != VSPEC_OK) return r;
     }
     const void *part = p->partial, *pcomp = p->partial_comp;
@@ -426,10 +426,10 @@ vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, 
         const void *k = p->npol == 2 ? (wide ? (const void *)reduce2048_kernel<2, 32, 1> : (const void *)reduce2048_kernel<2, 8, 4>)
                                      : (wide ? (const void *)reduce2048_kernel<1, 32, 1> : (const void *)reduce2048_kernel<1, 8, 4>);
         void *argsT[] = {&part, &groups, &stride, (void *)&N, (void *)&N2, &ia, &outp};
-        return launch(p, 2, spectra, k, dim3(N2 / 16 * 16 * (wide ? 4 : 16)), dim3(wide ? 256 : 512), argsT, 0, st);
+        return launch(p, 2, spectra, k, dim3(N2 / 16 * 16 * (wide ? 4 : 16), nsub), dim3(wide ? 256 : 512), argsT, 0, st);
     }
     void *argsR[] = {&part, &groups, &stride, (void *)&N, (void *)&N1, (void *)&N2, &ia, &ib, &outp};
-    return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32), dim3(32, 8), argsR, 0, st);
+    return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32, nsub), dim3(32, 8), argsR, 0, st);
 }
 
 const void *pick_kernel_fused(int logn1, int pt) {
@@ -1158,6 +1158,7 @@ vspec_status vspec_plan_create_shaped(vspec_plan **out, int nchan, int ntaps, in
 
 static bool sb_in_place(const vspec_plan *p, int nsub);
 static vspec_plan *sb_plan(vspec_plan *p);
+static int band_slots(const vspec_plan *p, int nsub, int nB);
 
 vspec_status vspec_plan_create_sb(vspec_plan **out, int nchan, int ntaps, int npol, int nsub,
                                   vspec_mode mode, vspec_window window, unsigned flags) {
@@ -1172,7 +1173,28 @@ vspec_status vspec_plan_create_sb(vspec_plan **out, int nchan, int ntaps, int np
     if (st != VSPEC_OK || nsub == 1) return st;
     vspec_plan *p = *out;
     p->nsub = nsub;
-    if (sb_in_place(sb_plan(p), nsub)) return VSPEC_OK;  // kernel A reads each band in place: no de-interleave scratch
+    if (vspec_plan *t = sb_plan(p); sb_in_place(t, nsub)) {
+        // kernel A reads each band in place: no de-interleave scratch, but
+        // partial sums for every band of the default launch
+        const int need = band_slots(t, nsub, t->num_sms * t->occB);
+        if (need > t->slots_cap) {
+            const size_t per = (size_t)t->N * sizeof(float4);
+            size_t tot = 0;
+            cudaFree(t->partial);
+            t->partial = nullptr;
+            st = dev_alloc(&t->partial, need * per, &tot);
+            if (st != VSPEC_OK) {
+                free_plan(p);
+                *out = nullptr;
+                return st;
+            }
+            const size_t more = (size_t)(need - t->slots_cap) * per;
+            t->slots_cap = need;
+            t->scratch_bytes += more;
+            if (t != p) p->scratch_bytes += more;
+        }
+        return VSPEC_OK;
+    }
     const int Peff = mode == VSPEC_PFB ? ntaps : 1;
     const size_t per_spec = (size_t)nchan * npol * 2;  // bytes of one sub-band per spectrum
     p->sb_chunk = (int)std::max<size_t>(1, (64u << 20) / (per_spec * nsub));
@@ -1404,23 +1426,30 @@ static void make_params(const vspec_plan *p, const int8_t *d_in, int nspectra, v
                         vspec::RowParams &cb);
 
 // Whether every band of a sub-band call fits one kernel-A and one kernel-B
-// launch per chunk (run_bands): the tiled fold, the slots of nsub bands
-// within the plan's partial sums, at least one spectrum of every band in the
-// chunk scratch.
+// launch per chunk (run_bands): the slots of nsub bands within the plan's
+// partial sums (vspec_plan_create_sb makes them large enough for the default
+// launch), at least one spectrum of every band in the chunk scratch.
+static int band_slots(const vspec_plan *p, int nsub, int nB) { return (nB / (nsub * (p->N2 / p->RB)) + 2) * nsub; }
 static bool bands_fit(const vspec_plan *p, int nsub) {
-    if (!sb_in_place(p, nsub) || !p->fold2048 || p->sc_alloc < nsub) return false;
-    const int nB = p->blocks_b > 0 ? p->blocks_b : p->num_sms * p->occB;
-    const int tilesB = nsub * (p->N2 / p->RB);
-    return (nB / tilesB + 2) * nsub <= p->slots_cap;
+    if (!sb_in_place(p, nsub) || p->sc_alloc < nsub) return false;
+    return band_slots(p, nsub, p->blocks_b > 0 ? p->blocks_b : p->num_sms * p->occB) <= p->slots_cap;
 }
 
 // Every band of a sub-band call in one kernel-A and one kernel-B launch per
-// chunk. Kernel A's tile X is column tile X / nsub of band X mod nsub, so
-// adjacent tiles (whose CTAs run together) read the same input lines and the
-// input comes from HBM once. A spectrum's intermediate holds the bands one
+// chunk. With a power-of-two nsub a kernel-A tile is C consecutive words of
+// the interleaved rows (C / nsub columns of every band), staged with 16-byte
+// copies like plain input (8 x 4096 channels, 501 spectra: 548 -> 179 us with
+// one launch set for all bands; 8 x 32768, 125 spectra: kernel A 333 -> 223
+// us). Otherwise, and where more than two bands would leave a band fewer than
+// kSbTileCols columns of a tile (its scratch runs are then a sector or less:
+// kernel A at 8 x 65536 421 us gathered, 521 us interleaved; with two bands
+// at 262144 channels 335 gathered, 286 interleaved), tile X is column tile X / nsub of band X mod nsub, gathered with
+// 4-byte copies: adjacent tiles (whose CTAs run together) read the same input
+// lines, so the input still comes from HBM once. A spectrum's intermediate holds the bands one
 // after another, a virtual spectrum of nsub N points whose nsub N2 rows kernel
 // B transforms as usual; the partial sums are slots of that virtual spectrum,
-// and one fold per band reads its part.
+// and one fold launch covers every band.
+constexpr int kSbTileCols = 4;
 static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int nspectra, float *d_accum,
                               cudaStream_t st) {
     const int nA = p->blocks_a > 0 ? p->blocks_a : p->num_sms * p->occA;
@@ -1438,6 +1467,7 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
     ca.nsub = nsub;
     ca.band = -1;
     ca.zstride = NV;
+    if (is_pow2(nsub) && (p->C / nsub >= kSbTileCols || nsub == 2)) ca.lsub = ilog2(nsub);
     ca.tiles = nsub * (p->N1 / p->C);
     cb.N = (int)NV;
     cb.tiles = tilesB;
@@ -1460,21 +1490,7 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
         r = launch(p, 1, sc * nsub, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st);
         if (r != VSPEC_OK) return r;
     }
-    // one tiled fold per band: its positions are [b N, (b + 1) N) of every slot
-    using namespace vspec;
-    const int N2 = p->N2, Nv = (int)NV, groups = slots, stride = 1;
-    const bool wide = N2 >= 64;
-    const void *k = wide ? (const void *)reduce2048_kernel<2, 32, 1> : (const void *)reduce2048_kernel<2, 8, 4>;
-    const int *ia = p->invA;
-    for (int b = 0; b < nsub; b++) {
-        const void *part = reinterpret_cast<const float4 *>(p->partial) + (size_t)b * p->N;
-        void *outp = d_accum + (size_t)b * p->N * 4;
-        void *argsT[] = {&part, (void *)&groups, (void *)&stride, (void *)&Nv, (void *)&N2, &ia, &outp};
-        vspec_status r = launch(p, 2, nspectra, k, dim3(N2 / 16 * 16 * (wide ? 4 : 16)), dim3(wide ? 256 : 512),
-                                argsT, 0, st);
-        if (r != VSPEC_OK) return r;
-    }
-    return VSPEC_OK;
+    return launch_fold(p, slots, d_accum, nspectra, st, nsub);
 }
 
 vspec_status vspec_execute(vspec_plan *plan, const int8_t *d_in, int nspectra, float *d_accum,

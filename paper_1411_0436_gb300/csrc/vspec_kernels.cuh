@@ -88,8 +88,10 @@ struct ColParams {
     // sub-band input read in place (register-column kernels): sample m of band
     // b is word m nsub + b of the input, [time][sub][pol]; nsub = 1: plain.
     // band = -1: every band in one launch, tile X being tile X / nsub of band
-    // X mod nsub, band b's spectra at Z + b N with a spectrum stride of zstride
-    int nsub = 1, band = 0;
+    // X mod nsub, band b's spectra at Z + b N with a spectrum stride of zstride.
+    // lsub > 0 (band = -1, nsub = 2^lsub): a tile is C consecutive words of the
+    // interleaved rows instead, word w being column w / nsub of band w mod nsub
+    int nsub = 1, band = 0, lsub = 0;
     long long zstride = 0;  // scratch elements per spectrum (0: N)
 };
 
@@ -527,15 +529,19 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
     const int t = threadIdx.x;                                         // point n2 * C + c
     const int D = PT - p.P;                                            // leading zero taps
     const size_t zs = p.zstride > 0 ? (size_t)p.zstride : (size_t)p.N;  // scratch spectrum stride
+    // this thread's column (its points and butterflies all have c = t mod C) and band
+    const int w0 = x * C, n1t = (w0 + t % C) >> p.lsub;
+    if (p.lsub) {
+        band = (w0 + t % C) & (p.nsub - 1);
+        Zc = reinterpret_cast<P2 *>(Zc) + (size_t)band * p.N;
+    }
     // first-pass twiddles W_N2^(j q) (ordered before use by the loop's barriers)
     if (load_twc)
         for (int e = t; e < G::TWC; e += PTS) twc[e] = __ldg(p.twA + p.pass[0].off + e);
     {
-        const int n1_0 = x * C;
-        for (int e = t; e < PTS; e += PTS)  // W_N^(n1 k2), k2 = pos
-            tws[G::twi(e / C, e % C)] = __ldg(p.twZ + (size_t)(e / C) * p.N1 + n1_0 + (e % C));
+        tws[G::twi(t / C, t % C)] = __ldg(p.twZ + (size_t)(t / C) * p.N1 + n1t);  // W_N^(n1 k2), k2 = pos
 
-        const long long n_pt = n1_0 + (t % C) + (long long)p.N1 * (t / C);
+        const long long n_pt = n1t + (long long)p.N1 * (t / C);
         // the tile's coefficients, read back for every batch so that their
         // registers are free during the column DFTs (each thread reads only
         // what it wrote: no barrier needed)
@@ -555,12 +561,12 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
         // (sub-band input: 4-byte copies of this band's samples, nsub words apart)
         auto stage = [&](int sb, int buf) {
             const int nbb = min(SPB, s_end - sb);
-            if (p.nsub > 1) {
+            if (p.nsub > 1 && !p.lsub) {
                 for (int e = t; e < nbb * PTS; e += PTS) {
                     const int u = e / PTS, r = e % PTS;  // r = n2 C + c
                     const long long fr = s0 + sb + u + p.P - 1;
                     const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) +
-                                          (fr * p.N + n1_0 + (long long)p.N1 * (r / C) + r % C) * p.nsub + band;
+                                          (fr * p.N + w0 + (long long)p.N1 * (r / C) + r % C) * p.nsub + band;
                     uint32_t *dst = raw + (buf * SPB + u) * PTS + r;
                     if (dbg_ok(fr < p.nframes, kDbgInput))
                         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
@@ -574,8 +580,8 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
                 const int u = e / per_frame, r = e % per_frame;
                 const int n2 = r / per_row, ch = r % per_row;
                 const long long fr = s0 + sb + u + p.P - 1;
-                const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) + fr * p.N + n1_0 +
-                                      (long long)p.N1 * n2 + ch * 4;
+                const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) +
+                                      ((fr * p.N + (long long)p.N1 * n2) << p.lsub) + w0 + ch * 4;
                 uint32_t *dst = raw + (buf * SPB + u) * PTS + n2 * C + ch * 4;
                 if (dbg_ok(fr < p.nframes, kDbgInput))
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
@@ -619,8 +625,8 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
 #pragma unroll
                         for (int q = 0; q < N2; q++) v[q] = data[sb * SS + q * C + c];
                         Dft<N2>::run(v);
-                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + n1_0 + c;
-                        if (!dbg_ok(s_base + sb < sc && n1_0 + c < p.N1, kDbgScratch)) continue;
+                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + n1t;
+                        if (!dbg_ok(s_base + sb < sc && n1t < p.N1, kDbgScratch)) continue;
                         z[0] = v[0];
 #pragma unroll
                         for (int q = 1; q < N2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[G::twi(q, c)]);
@@ -658,8 +664,8 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
                         for (int q = 0; q < R2; q++) v[q] = d[q * C];
                         Dft<R2>::run(v);
                         P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs +
-                                (size_t)(b * R2) * p.N1 + n1_0 + c;
-                        if (!dbg_ok(s_base + sb < sc && n1_0 + c < p.N1, kDbgScratch)) continue;
+                                (size_t)(b * R2) * p.N1 + n1t;
+                        if (!dbg_ok(s_base + sb < sc && n1t < p.N1, kDbgScratch)) continue;
 #pragma unroll
                         for (int q = 0; q < R2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[G::twi(b * R2 + q, c)]);
                     }
@@ -681,12 +687,12 @@ __global__ void __launch_bounds__(512, 1) fir_colreg_kernel(const __grid_constan
         const int s_beg = (int)(f - base);
         const int s_end = (int)(min(sp.hi, base + p.sc) - base);
         f = base + s_end;
-        if (p.band < 0) {  // every band in this launch: adjacent tiles are the bands of one column tile
+        if (p.band < 0 && !p.lsub) {  // every band in this launch: adjacent tiles are the bands of one column tile
             const int band = x % p.nsub;
             colreg_tile<N2, R1>(p, reinterpret_cast<P2 *>(p.Z) + (size_t)band * p.N, p.s0, p.sc, x / p.nsub, s_beg,
                                 s_end, smem_raw, first, band);
         } else {
-            colreg_tile<N2, R1>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.band);
+            colreg_tile<N2, R1>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.lsub ? 0 : p.band);
         }
         first = false;
     }
@@ -734,6 +740,10 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
     float *wins = reinterpret_cast<float *>(twc + G::TWC);                         // [N2][C]
     const int t = threadIdx.x;
     const size_t zs = p.zstride > 0 ? (size_t)p.zstride : (size_t)p.N;  // scratch spectrum stride
+    // the tile's first word of a row; word w is column w / nsub of band w mod nsub (lsub > 0)
+    const int w0 = x * C;
+    auto column = [&](int c) { return (w0 + c) >> p.lsub; };
+    auto zcol = [&](int c) { return (p.lsub ? (size_t)((w0 + c) & (p.nsub - 1)) * p.N : 0) + column(c); };
     if (load_twc)
         for (int e = t; e < G::TWC; e += 512) twc[e] = __ldg(p.twA + p.pass[0].off + e);
     // sample (pos e of the tile) of spectrum row rb, times the window value when there is one
@@ -746,21 +756,20 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
         return v;
     };
     {
-        const int n1_0 = x * C;
         for (int e = t; e < PTS; e += 512) {  // W_N^(n1 k2(pos)); window values h[n1 + N1 n2]
-            tws[e] = __ldg(p.twZ + (size_t)(e / C) * p.N1 + n1_0 + (e % C));
-            if (p.win) wins[e] = __ldg(p.coef + (size_t)(e / C) * p.N1 + n1_0 + (e % C));
+            tws[e] = __ldg(p.twZ + (size_t)(e / C) * p.N1 + column(e % C));
+            if (p.win) wins[e] = __ldg(p.coef + (size_t)(e / C) * p.N1 + column(e % C));
         }
         // frames of SPB spectra into raw[buf], 16-byte copies (sub-band input:
         // 4-byte copies of this band's samples, nsub words apart)
         auto stage = [&](int sb, int buf) {
             const int nbb = min(SPB, s_end - sb);
-            if (p.nsub > 1) {
+            if (p.nsub > 1 && !p.lsub) {
                 for (int e = t; e < nbb * PTS; e += 512) {
                     const int u = e / PTS, r = e % PTS;  // r = n2 C + c
                     const long long fr = s0 + sb + u;
                     const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) +
-                                          (fr * p.N + n1_0 + (long long)p.N1 * (r / C) + r % C) * p.nsub + band;
+                                          (fr * p.N + w0 + (long long)p.N1 * (r / C) + r % C) * p.nsub + band;
                     uint32_t *dst = raw + (buf * SPB + u) * PTS + r;
                     if (dbg_ok(fr < p.nframes, kDbgInput))
                         asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
@@ -774,8 +783,8 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
                 const int u = e / per_frame, r = e % per_frame;
                 const int n2 = r / per_row, ch = r % per_row;
                 const long long fr = s0 + sb + u;
-                const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) + fr * p.N + n1_0 +
-                                      (long long)p.N1 * n2 + ch * 4;
+                const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) +
+                                      ((fr * p.N + (long long)p.N1 * n2) << p.lsub) + w0 + ch * 4;
                 uint32_t *dst = raw + (buf * SPB + u) * PTS + n2 * C + ch * 4;
                 if (dbg_ok(fr < p.nframes, kDbgInput))
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
@@ -800,8 +809,8 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
 #pragma unroll
                         for (int q = 0; q < N2; q++) v[q] = sample(rb + sb * PTS, q * C + c);
                         Dft<N2>::run(v);
-                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + n1_0 + c;
-                        if (!dbg_ok(s_base + sb < sc && n1_0 + c < p.N1, kDbgScratch)) continue;
+                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + zcol(c);
+                        if (!dbg_ok(s_base + sb < sc && column(c) < p.N1, kDbgScratch)) continue;
                         z[0] = v[0];
 #pragma unroll
                         for (int q = 1; q < N2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[q * C + c]);
@@ -838,8 +847,8 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
                         for (int q = 0; q < R2; q++) v[q] = d[q * C];
                         Dft<R2>::run(v);
                         P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs +
-                                (size_t)(b * R2) * p.N1 + n1_0 + c;
-                        if (!dbg_ok(s_base + sb < sc && n1_0 + c < p.N1, kDbgScratch)) continue;
+                                (size_t)(b * R2) * p.N1 + zcol(c);
+                        if (!dbg_ok(s_base + sb < sc && column(c) < p.N1, kDbgScratch)) continue;
 #pragma unroll
                         for (int q = 0; q < R2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[(b * R2 + q) * C + c]);
                     }
@@ -861,12 +870,12 @@ __global__ void __launch_bounds__(512) fir_coldir_kernel(const __grid_constant__
         const int s_beg = (int)(f - base);
         const int s_end = (int)(min(sp.hi, base + p.sc) - base);
         f = base + s_end;
-        if (p.band < 0) {  // every band in this launch: adjacent tiles are the bands of one column tile
+        if (p.band < 0 && !p.lsub) {  // every band in this launch: adjacent tiles are the bands of one column tile
             const int band = x % p.nsub;
             coldir_tile<N2>(p, reinterpret_cast<P2 *>(p.Z) + (size_t)band * p.N, p.s0, p.sc, x / p.nsub, s_beg, s_end,
                             smem_raw, first, band);
         } else {
-            coldir_tile<N2>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.band);
+            coldir_tile<N2>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.lsub ? 0 : p.band);
         }
         first = false;
     }
@@ -1670,7 +1679,7 @@ __global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, in
     const int k2_0 = 16 * (blockIdx.x % nk);
     const int q1 = (blockIdx.x / nk) % 16, g = blockIdx.x / (nk * 16);
     const int p0 = 128 * q1 + PB * g;
-    const A *pp = reinterpret_cast<const A *>(partial);
+    const A *pp = reinterpret_cast<const A *>(partial) + (size_t)blockIdx.y * N;  // band blockIdx.y of every slot
     for (int e = threadIdx.x; e < E * L; e += blockDim.x) {
         const int l = e / E, r = (e % E) / PB, j = e % PB;
         const size_t idx = (size_t)__ldg(invA + k2_0 + r) * 2048 + p0 + j;
@@ -1688,7 +1697,7 @@ __global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, in
         tile[l][r][j] = s;
     }
     __syncthreads();
-    A *o = reinterpret_cast<A *>(out);
+    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N;
     for (int e = threadIdx.x; e < E; e += blockDim.x) {
         const int r = e & 15, j = e >> 4;  // position offset j = 8 (q2 - Q2G g) + q3
         const int k1 = q1 + 16 * (Q2G * g + (j >> 3)) + 256 * (j & 7);
@@ -1724,7 +1733,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const void *partial, int gr
     __shared__ A lane_sum[8][32];
     const int k = blockIdx.x * 32 + threadIdx.x;
     const int y = threadIdx.y;
-    const A *pp = reinterpret_cast<const A *>(partial);
+    const A *pp = reinterpret_cast<const A *>(partial) + (size_t)blockIdx.y * N;  // band blockIdx.y of every slot
     A s;
     if constexpr (NPOL == 2) s = make_float4(0.f, 0.f, 0.f, 0.f);
     else s = 0.f;
@@ -1744,7 +1753,7 @@ __global__ void __launch_bounds__(256) reduce_kernel(const void *partial, int gr
     lane_sum[y][threadIdx.x] = s;
     __syncthreads();
     if (y != 0 || k >= N) return;
-    A *o = reinterpret_cast<A *>(out);
+    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N;
 #pragma unroll
     for (int l = 1; l < 8; l++) {
         const A v = lane_sum[l][threadIdx.x];
