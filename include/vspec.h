@@ -327,7 +327,8 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  *   A=colreg|coldir|general|gather|none   kernel A's form: register columns
  *                            (dual-pol PFB), register columns (dual-pol
  *                            direct), the general kernel, taps read from the
- *                            input; none for one-row transforms
+ *                            input (gather-blocked: from frames staged in
+ *                            shared memory); none for one-row transforms
  *   B=row2048|general|tensor kernel B's form
  *   fir-in-B                 one-row transform: the FIR runs in kernel B
  *   kahan                    compensated accumulation

@@ -27,6 +27,7 @@
 #include "vspec_kernels_tcfir.cuh"
 #include "vspec_ring.cuh"
 #include "vspec_row2048.cuh"
+#include "vspec_colblk.cuh"
 #include "vspec_bp.cuh"
 #include "vspec_internal.h"
 
@@ -714,6 +715,12 @@ vspec_status build_plan(vspec_plan *p) {
     const bool colreg_tiles = p->npol == 2 && pfb && PT == 8 && !p->gather && (N1 == 2048 || N1 == 4096) && N2 >= 2 &&
                               N2 <= 128 && !p->req_cols;
     if (colreg_tiles) C = 512 / N2;
+    // dual-pol PFB too long for a register window, 512-point columns (2^20):
+    // the blocked kernel A, up to its 8 taps (0.78 against 1.77 ms per 100
+    // spectra; the gather kernel keeps 9 .. 16 taps and single polarisation)
+    const bool colblk = p->npol == 2 && p->gather && p->P <= vspec::ColBlk::PT && N2 == vspec::ColBlk::N2 &&
+                        N1 >= vspec::ColBlk::C && !p->req_cols;
+    if (colblk) C = vspec::ColBlk::C;
     if (p->req_cols) {  // a requested tile width: the general kernel A
         const int c = p->req_cols;
         if (!is_pow2(c) || c < cmin || c > N1 || (long long)c * N2 > 4096 || N2 == 1) {
@@ -724,7 +731,7 @@ vspec_status build_plan(vspec_plan *p) {
     }
     const int pts = N2 * C;
     const int TA = std::min(512, pts);
-    const int PPT = pts / TA;
+    const int PPT = colblk ? 1 : pts / TA;
     p->N1 = N1;
     p->N2 = N2;
     p->C = C;
@@ -741,6 +748,10 @@ vspec_status build_plan(vspec_plan *p) {
         p->formA = "coldir";
     }
     if (p->gather) p->formA = "gather";
+    if (colblk) {
+        p->kernelA = (const void *)vspec::fir_colblk_kernel;
+        p->formA = "gather-blocked";
+    }
     if (!p->kernelA) {
         g_last_error = "no kernel instance for this tap count and size";
         return VSPEC_ERR_UNSUPPORTED;
@@ -804,7 +815,7 @@ vspec_status build_plan(vspec_plan *p) {
     // sums or tensor-core rows: four radix-8 passes (row4096_kernel)
     const bool row4096 = N1 == 4096 && p->npol == 2 && !p->fir_b &&
                          !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8));
-    const std::vector<int> rA = (tcfir || coltc) ? std::vector<int>{N2} : colreg ? r_colreg : coldir ? r_coldir
+    const std::vector<int> rA = colblk ? std::vector<int>{8, 8, 8} : (tcfir || coltc) ? std::vector<int>{N2} : colreg ? r_colreg : coldir ? r_coldir
                                                                                : radix_list(e2, maxbitsA),
                            rB = row4096 ? std::vector<int>{8, 8, 8, 8} : radix_list(e1);
     int twA_n = 0, twB_n = 0;
@@ -847,6 +858,7 @@ vspec_status build_plan(vspec_plan *p) {
     p->smemA = (size_t)PT * N2 * C * elem + (size_t)N2 * C * sizeof(float2) +
                (!p->gather ? 2 * (size_t)PT * N2 * C * p->npol * 2 : 0);
     if (colreg) p->smemA = smem_colreg;
+    if (colblk) p->smemA = vspec::ColBlk::smem;
     if (tcfir || coltc) p->smemA = smem_tcA;
     if (coldir) p->smemA = smem_coldir;
     p->smemB = (size_t)p->RB * (N1 + (N1 >> 4)) * elem + (size_t)p->RB * N1 * accel;
