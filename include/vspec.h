@@ -329,7 +329,8 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  *                            direct), the general kernel, taps read from the
  *                            input (gather-blocked: from frames staged in
  *                            shared memory); none for one-row transforms
- *   B=row2048|general|tensor kernel B's form
+ *   B=row2048|general|tensor kernel B's form (-batched: the one-row kernel of
+ *                            512, 1024 and 2048 channels)
  *   fir-in-B                 one-row transform: the FIR runs in kernel B
  *   kahan                    compensated accumulation
  * Writes at most len bytes including the terminating NUL (truncating).
@@ -376,9 +377,10 @@ VSPEC_API vspec_status vspec_plan_kernel_stats(vspec_plan *plan, int kind, int r
  *   blocks_a         CTAs per kernel-A launch: 0 (one wave, the default) or
  *                    1 .. limit.blocks_a
  *   blocks_b         CTAs per kernel-B launch: 0 (one wave) or 1 .. limit.blocks_b
- * One-pass fused plans (dual-pol, 2048..32768 channels) run clusters of CTAs.
- * Except at 2048 channels they own a two-kernel plan of the same problem,
- * which the three fields above tune, and use it in two ways:
+ * One-pass fused plans (dual-pol, 2048..32768 channels) run clusters of CTAs,
+ * or at 2048 channels single CTAs. Except at 2048 channels they own a
+ * two-kernel plan of the same problem, which the three fields above tune, and
+ * use it in two ways:
  *   two_kernel_from  a call with at least this many spectra runs wholly on
  *                    the two-kernel path (faster on long calls: its work is
  *                    spread over every SM); 0 .. INT_MAX, INT_MAX: never. The

@@ -36,6 +36,10 @@ using vspec::Pass;
 // vspec_ring.cu
 const void *vspec_pick_kernel_ring(int N2, size_t *smem);
 cudaError_t vspec_ring_debug_flags(unsigned *flags, bool clear);
+// vspec_rowbatch.cu
+const void *vspec_pick_kernel_rowbatch(int nchan, int npol, int P, size_t *smem);
+const void *vspec_pick_fold_row(int npol);
+cudaError_t vspec_rowbatch_debug_flags(unsigned *flags, bool clear);
 // vspec_bp.cu
 const void *vspec_bp_kernel();
 size_t vspec_bp_smem_a(int form, int N2);
@@ -166,6 +170,11 @@ struct vspec_plan {
     // fused plans: a two-kernel plan that channelizes a share of the spectra
     // on the SMs the clusters leave idle, concurrently with the fused kernel
     vspec_plan *assist = nullptr;
+    // 2048 channels: the one-row plan that runs every call. One CTA holds the
+    // whole transform there, and row_batch_kernel is faster than the cluster
+    // kernel was at every length (PFB, us per call: 10 spectra 18.5 -> 16.4,
+    // 1000 39 -> 27, 4096 103 -> 64; direct 4096 91 -> 47)
+    vspec_plan *row_plan = nullptr;
     vspec_plan *owner = nullptr;  // the plan whose profiling records this plan's launches
     int assist_permille = 0;
     int two_kernel_from = INT_MAX;  // fused plans: calls with this many spectra use `assist` alone
@@ -183,6 +192,7 @@ struct vspec_plan {
     int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel (in twB's allocation)
     float2 *twBt = nullptr;      // its twiddles (in twB's allocation)
     bool row_groups = false;     // kernel B is row2048_group_kernel
+    bool row_batch = false;      // kernel B is row_batch_kernel (one-row transforms)
     // persistent ring form (VSPEC_PLAN_RING): Z holds ringR slots of ringS
     // spectra, `partial` ring_sets partial-sum sets
     bool ring = false;
@@ -400,6 +410,13 @@ vspec_status launch(vspec_plan *p, int kind, int spectra, const void *fn, dim3 g
 vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, cudaStream_t st, int nsub = 1) {
     int groups = slots, stride = nsub;  // a slot holds the nsub bands one after another
     const int N = p->N, N1 = p->N1, N2 = p->N2;
+    if (p->row_batch) {
+        const void *part = p->partial;
+        int n = N, R1 = p->passB[0].r, R2 = p->passB[1].r;
+        void *outp = d_accum;
+        void *args[] = {&part, &slots, &n, &R1, &R2, &outp};
+        return launch(p, 2, spectra, vspec_pick_fold_row(p->npol), dim3(N / 8), dim3(8, 64), args, 0, st);
+    }
     if (slots > 128) {
         groups = (slots + 15) / 16;
         stride = 16 * nsub;
@@ -436,8 +453,6 @@ vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, 
 const void *pick_kernel_fused(int logn1, int pt) {
     using namespace vspec::fused;
     switch (logn1 * 100 + pt) {
-        case 401: return (const void *)fused_kernel<4, 1>;
-        case 408: return (const void *)fused_kernel<4, 8>;
         case 501: return (const void *)fused_kernel<5, 1>;
         case 508: return (const void *)fused_kernel<5, 8>;
         case 601: return (const void *)fused_kernel<6, 1>;
@@ -480,6 +495,7 @@ void free_plan(vspec_plan *p) {
         cudaEventDestroy(p->ev_main);
         cudaEventDestroy(p->ev_assist);
     }
+    if (p->row_plan) free_plan(p->row_plan);
     for (cudaEvent_t e : p->event_pool) cudaEventDestroy(e);
     release_host_pipeline(p);
     cudaFree(p->coef);
@@ -558,7 +574,8 @@ void ring_default_shape(vspec_plan *p) {
 }
 constexpr int kRowElems = 2048;  // target row-DFT elements per kernel-B CTA
 
-// Fused one-pass plan: dual-pol, 2048..32768 channels, 8-tap PFB or direct.
+// Fused one-pass plan: dual-pol, 2048..32768 channels, 8-tap PFB or direct
+// (the cluster kernel above 2048 channels).
 vspec_status build_fused_plan(vspec_plan *p) {
     namespace F = vspec::fused;
     namespace W = vspec::fusedw;
@@ -573,6 +590,12 @@ vspec_status build_fused_plan(vspec_plan *p) {
     p->N2 = N2;
     p->cluster = N1 / F::kCols;
     p->kernelR = (const void *)vspec::reduce_kernel<2>;
+    if (p->cluster == 1) {  // 2048 channels: the one-row plan runs the calls (setup_assist creates it)
+        VSPEC_CUDA(cudaGetDevice(&p->device));
+        VSPEC_CUDA(cudaDeviceGetAttribute(&p->num_sms, cudaDevAttrMultiProcessorCount, p->device));
+        p->nclusters = p->num_sms;
+        return VSPEC_OK;
+    }
     std::vector<int> rA, rB;
     if (p->fused_w) {
         p->kernelF = PT == 8 ? (const void *)W::fused_w_kernel<8> : (const void *)W::fused_w_kernel<1>;
@@ -892,6 +915,23 @@ vspec_status build_plan(vspec_plan *p) {
         p->formB = "row2048";
         p->fold2048 = N2 >= 16 && !p->kahan;
     }
+    // one-row transforms of 512 .. 2048 channels: the batched one-pass kernel
+    // (1024 channels dual-pol, 8 taps, 2048 spectra: 59 us in the general row
+    // kernel; compensated plans, and dual-pol 2048 channels with more than 8
+    // taps, keep the kernels above)
+    const void *kernelB_limits = p->kernelB;  // the kernel whose occupancy sets the launch limits
+    const int TB_limits = p->TB;
+    const size_t smem_limits = p->smemB;
+    if (p->fir_b && !p->kahan) {
+        size_t smem = 0;
+        if (const void *k = vspec_pick_kernel_rowbatch(N, p->npol, p->P, &smem)) {
+            p->row_batch = true;
+            p->kernelB = k;
+            p->TB = 512;
+            p->smemB = smem;
+            p->formB = N == 2048 ? "row2048-batched" : "general-batched";
+        }
+    }
     // 4096-point rows (radix 8, 8, 8, 8): one spectrum per pass sequence,
     // register accumulators
     if (row4096 && !p->tc && p->RB == 1 && p->passB.size() == 4) {
@@ -943,8 +983,14 @@ vspec_status build_plan(vspec_plan *p) {
     p->sc_max = std::min({p->sc_cap, kMaxChunkSpectra, (int)std::max<size_t>(1, kScratchBudget / per_spec)});
     if (p->fir_b) p->sc_cap = p->sc_max = kMaxChunkSpectra;  // launch length only: no scratch
     // partial-sum slots for the largest kernel-B launch a tuning may ask for
-    // (row2048_group_kernel runs one CTA per SM, but keeps the limits of two)
+    // (row2048_group_kernel and row_batch_kernel run one CTA per SM, but keep
+    // the limits of the kernels that run the other plans of their sizes)
     p->maxB = p->row_groups ? std::max(2, p->occB) : p->occB;
+    if (p->row_batch) {
+        VSPEC_CUDA(raise_smem_cap(kernelB_limits, smem_limits));
+        VSPEC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->maxB, kernelB_limits, TB_limits, smem_limits));
+        p->maxB = std::max(p->maxB, p->occB);
+    }
     p->slots_cap = slots_for(p, kMaxWaves * p->num_sms * p->maxB);
 
     // device tables and scratch
@@ -954,10 +1000,12 @@ vspec_status build_plan(vspec_plan *p) {
     if ((st = dev_alloc((void **)&p->coef, sizeof(float) * (size_t)Lc, &tot))) return st;
     if ((st = dev_alloc((void **)&p->twA, sizeof(float2) * (size_t)std::max(1, twA_n), &tot))) return st;
     // with the row kernel's own twiddle order and wait flag after the table
-    const int twBt_n = p->row_groups ? vspec::Row2048::TW1 + vspec::Row2048::TW2 : 0;
+    const bool own_tw = p->row_groups || p->row_batch;
+    const int tw1_n = own_tw ? p->passB[0].m * (p->passB[0].r - 1) : 0;
+    const int twBt_n = own_tw ? tw1_n + p->passB[1].m * (p->passB[1].r - 1) : 0;
     if ((st = dev_alloc((void **)&p->twB, sizeof(float2) * (size_t)(std::max(1, twB_n) + twBt_n + 1), &tot))) return st;
+    if (own_tw) p->twBt = p->twB + twB_n;
     if (p->row_groups) {
-        p->twBt = p->twB + twB_n;
         p->row_status = reinterpret_cast<int *>(p->twBt + twBt_n);
         VSPEC_CUDA(cudaMemset(p->row_status, 0, sizeof(int)));
     }
@@ -1013,9 +1061,9 @@ vspec_status build_plan(vspec_plan *p) {
         for (const Pass &ps : p->passB)
             if (ps.m * (ps.r - 1) > 0)
                 vspec::gen_pass_tw_kernel<<<(ps.m * (ps.r - 1) + 255) / 256, 256, 0, s0>>>(p->twB, ps);
-        if (p->row_groups) {
-            vspec::gen_pass_tw_t_kernel<<<(vspec::Row2048::TW1 + 255) / 256, 256, 0, s0>>>(p->twBt, p->passB[0]);
-            vspec::gen_pass_tw_t_kernel<<<1, 256, 0, s0>>>(p->twBt + vspec::Row2048::TW1, p->passB[1]);
+        if (own_tw) {
+            vspec::gen_pass_tw_t_kernel<<<(tw1_n + 255) / 256, 256, 0, s0>>>(p->twBt, p->passB[0]);
+            vspec::gen_pass_tw_t_kernel<<<1, 256, 0, s0>>>(p->twBt + tw1_n, p->passB[1]);
         }
         vspec::gen_twz_kernel<<<(N + 255) / 256, 256, 0, s0>>>(p->twZ, N, N1, N2, d_kA);
         if (p->tc_cols && !p->tc_int8) {
@@ -1067,8 +1115,8 @@ vspec_status vspec_plan_create(vspec_plan **out, int nchan, int ntaps, int npol,
 // and hides its memory latency better, and beyond a per-size number of
 // spectra it is the faster path; below it the fused kernel's smaller fixed
 // cost wins. The thresholds come from measurements on GB300 (both paths
-// timed at 50 to 4000 spectra per call); at 2048 channels the fused path is
-// faster at every length.
+// timed at 50 to 4000 spectra per call). At 2048 channels the transform is one
+// row, and a one-row plan (row_plan) runs every call instead.
 // (2) Assist: on a device whose SM count is not a multiple of the cluster
 // size, the two-kernel plan can channelize a share of a call's spectra on
 // the SMs the clusters leave idle, concurrently with the fused kernel. The
@@ -1091,6 +1139,14 @@ static vspec_status setup_assist(vspec_plan *p) {
     const int busy = p->cluster * p->nclusters;
     const int idle = p->num_sms - busy;
     const int lg = ilog2(p->N) - 11;
+    if (lg == 0) {  // 2048 channels
+        vspec_status st = vspec_plan_create_ex(&p->row_plan, p->N, p->mode == VSPEC_PFB ? p->P : 1, p->npol,
+                                               (vspec_mode)p->mode, (vspec_window)p->window, VSPEC_PLAN_TWO_KERNEL);
+        if (st != VSPEC_OK) return st;
+        p->row_plan->owner = p;
+        p->scratch_bytes += p->row_plan->scratch_bytes;
+        return VSPEC_OK;
+    }
     p->two_kernel_from = (lg >= 0 && lg < 5) ? kTwoKernelFrom[p->mode == VSPEC_PFB ? 0 : 1][lg] : INT_MAX;
     if (idle < kAssistMinSms && p->two_kernel_from == INT_MAX) return VSPEC_OK;
     vspec_plan *a = nullptr;
@@ -1259,6 +1315,7 @@ vspec_status vspec_plan_describe(const vspec_plan *plan, char *buf, size_t len) 
     if (plan->fused) {
         d = "fused K=" + std::to_string(plan->cluster);
         if (plan->assist) d += " | " + two_kernel(plan->assist);
+        if (plan->row_plan) d += " | " + two_kernel(plan->row_plan);
     } else {
         d = two_kernel(plan);
     }
@@ -1705,7 +1762,9 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
         vspec::TcStatus ts{p->tc_status, g_wait_limit.load()};
         void *argsB[] = {&cb, &ts};
         const int gb = (int)std::min<long long>(nB, (long long)cb.tiles * sc);
-        r = launch(p, 1, sc, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st);
+        // (a 2048-channel plan reports its one-pass kernel as such)
+        const int kind = p->owner && p->owner->row_plan == p ? 3 : 1;
+        r = launch(p, kind, sc, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st);
         if (r != VSPEC_OK) return r;
     }
     if (before_fold) VSPEC_CUDA(cudaStreamWaitEvent(st, before_fold, 0));
@@ -1773,7 +1832,7 @@ static int bp_form(const vspec_plan *p0, const char **why) {
     int f = -1;
     if (p->npol != 2 || p->fused || p->kahan || p->tc || p->tc_cols || p->ring || p0->nsub != 1)
         w = "needs a dual-pol two-kernel FP32 plan (VSPEC_PLAN_TWO_KERNEL) without sub-bands";
-    else if (p->fir_b && p->N == 2048 && std::strcmp(p->formB, "row2048") == 0)
+    else if (p->fir_b && p->N == 2048)
         f = vspec::kBpRow2048Fir;
     else if (p->fir_b && p->N <= 1024 && p->P <= 8 && p->RB == 1)
         f = vspec::kBpRowFir;
@@ -1894,6 +1953,7 @@ static vspec_status execute_one(vspec_plan *p, const int8_t *d_in, int nspectra,
                                 cudaStream_t st) {
     if (p->ring) return run_ring(p, d_in, nspectra, d_accum, st);
     if (!p->fused) return run_two_kernel(p, d_in, nspectra, d_accum, st, nullptr);
+    if (p->row_plan) return run_two_kernel(p->row_plan, d_in, nspectra, d_accum, st, nullptr);
     if (p->assist && nspectra >= p->two_kernel_from)
         return run_two_kernel(p->assist, d_in, nspectra, d_accum, st, nullptr);
     const int sa = p->assist ? (int)((long long)nspectra * p->assist_permille / 1000) : 0;
@@ -2078,10 +2138,11 @@ vspec_status vspec_debug_flags(unsigned *flags, int clear) {
         const unsigned zero = 0;
         VSPEC_CUDA(cudaMemcpyToSymbol(vspec::g_debug_flags, &zero, sizeof(unsigned)));
     }
-    unsigned ring_flags = 0, bp_flags = 0;  // the ring and multi-bank kernels' own words
+    unsigned ring_flags = 0, bp_flags = 0, row_flags = 0;  // the other translation units' own words
     VSPEC_CUDA(vspec_ring_debug_flags(&ring_flags, clear != 0));
     VSPEC_CUDA(vspec_bp_debug_flags(&bp_flags, clear != 0));
-    *flags |= ring_flags | bp_flags;
+    VSPEC_CUDA(vspec_rowbatch_debug_flags(&row_flags, clear != 0));
+    *flags |= ring_flags | bp_flags | row_flags;
     return VSPEC_OK;
 #else
     (void)flags;

@@ -228,6 +228,7 @@ __device__ __forceinline__ void fill_w16(float2 *w16) {
     }
 }
 
+#ifndef VSPEC_NO_PLAN_TABLES  // defined in one translation unit
 // Batched 16-point DFTs, y[b][k] = sum_n x[b][n] W_16^(nk), 128 rows per CTA,
 // `terms` = 1 (X_hi F_hi) or 3 (hi/lo split). *status is set to 1 if the
 // wait for the tensor cores gives up after wait_limit polls; the CTA then
@@ -292,6 +293,7 @@ __global__ void __launch_bounds__(128) dft16_kernel(const float2 *x, float2 *y, 
         asm volatile("tcgen05.dealloc.cta_group::1.sync.aligned.b32 %0, %1;" :: "r"(tmem), "r"(32u) : "memory");
     }
 }
+#endif  // VSPEC_NO_PLAN_TABLES
 
 }  // namespace tc
 }  // namespace vspec
