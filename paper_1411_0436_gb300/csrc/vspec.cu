@@ -36,6 +36,9 @@ using vspec::Pass;
 // vspec_ring.cu
 const void *vspec_pick_kernel_ring(int N2, size_t *smem);
 cudaError_t vspec_ring_debug_flags(unsigned *flags, bool clear);
+// vspec_colgrp8.cu
+const void *vspec_pick_kernel_colgrp8(int N2, size_t *smem, int *groups);
+cudaError_t vspec_colgrp8_debug_flags(unsigned *flags, bool clear);
 // vspec_rowbatch.cu
 const void *vspec_pick_kernel_rowbatch(int nchan, int npol, int P, size_t *smem);
 const void *vspec_pick_fold_row(int npol);
@@ -191,6 +194,7 @@ struct vspec_plan {
     int *tc_status = nullptr;  // bounded-wait flag of the tensor-core or ring kernel
     int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel (in twB's allocation)
     float2 *twBt = nullptr;      // its twiddles (in twB's allocation)
+    int groupsA = 1;             // independent groups per kernel-A CTA (fir_colgrp_kernel)
     bool row_groups = false;     // kernel B is row2048_group_kernel
     bool row_batch = false;      // kernel B is row_batch_kernel (one-row transforms)
     // persistent ring form (VSPEC_PLAN_RING): Z holds ringR slots of ringS
@@ -308,20 +312,31 @@ const void *pick_kernel_tcfir(int N2, int P, size_t *smem, int *terms) {
 }
 
 // register-column kernel A (dual-pol PFB, 8 taps, 512-point tiles) for N2 in
-// 2 .. 128 and its column pass list (one pass up to 16 points, then 8 x N2/8)
-const void *pick_kernel_colreg(int N2, size_t *smem, std::vector<int> *radices) {
+// 2 .. 128, its groups per CTA and its column pass list (one pass up to 16
+// points, then 8 x N2/8). Whole columns in registers keep the kernel with the
+// register FIR window (one 512-thread group, one barrier less per batch);
+// longer columns run four independent groups. Kernel A, GB300, window against
+// groups: N2 = 2 (4096 spectra) 65 / 67 us, 16 (1000) 138 / 141 us, 32 (1000)
+// 310 / 285 us, 64 (2048) 1321 / 1199 us, 128 (256) 473 / 410 us.
+const void *pick_kernel_colreg(int N2, size_t *smem, int *groups, std::vector<int> *radices) {
     using namespace vspec;
     *radices = N2 <= 16 ? std::vector<int>{N2} : std::vector<int>{8, N2 / 8};
+    *groups = 1;
     switch (N2) {
         case 2: *smem = ColReg<2>::smem; return (const void *)fir_colreg_kernel<2>;
         case 4: *smem = ColReg<4>::smem; return (const void *)fir_colreg_kernel<4>;
         case 8: *smem = ColReg<8>::smem; return (const void *)fir_colreg_kernel<8>;
         case 16: *smem = ColReg<16>::smem; return (const void *)fir_colreg_kernel<16>;
-        case 32: *smem = ColReg<32, 8>::smem; return (const void *)fir_colreg_kernel<32, 8>;
-        case 64: *smem = ColReg<64, 8>::smem; return (const void *)fir_colreg_kernel<64, 8>;
-        case 128: *smem = ColReg<128, 8>::smem; return (const void *)fir_colreg_kernel<128, 8>;
     }
-    return nullptr;
+    return vspec_pick_kernel_colgrp8(N2, smem, groups);
+}
+
+// Kernel-A CTAs of a launch of `items` (tile, spectrum) items: at most nA, no
+// more workers (groups) than items, whole tile groups.
+int grid_a(int nA, int groups, int tileG, long long items) {
+    long long w = std::min<long long>((long long)nA * groups, items);
+    w = std::max<long long>(tileG, w / tileG * tileG);
+    return (int)((w + groups - 1) / groups);
 }
 
 constexpr int kNumKinds = 4;
@@ -798,7 +813,7 @@ vspec_status build_plan(vspec_plan *p) {
     size_t smem_colreg = 0;
     std::vector<int> r_colreg;
     const void *colreg = p->npol == 2 && pfb && PT == 8 && PPT == 1 && !p->gather && N2 * C == 512 && !p->req_cols
-                             ? pick_kernel_colreg(N2, &smem_colreg, &r_colreg) : nullptr;
+                             ? pick_kernel_colreg(N2, &smem_colreg, &p->groupsA, &r_colreg) : nullptr;
     if (colreg) {
         p->kernelA = colreg;
         p->formA = "colreg";
@@ -819,6 +834,7 @@ vspec_status build_plan(vspec_plan *p) {
     }
     const void *coltc = !want_int8 && (p->flags & VSPEC_PLAN_TENSOR) && colreg && N1 == 2048
                             ? pick_kernel_coltc(N2, &smem_tcA) : nullptr;
+    if (tcfir || coltc) p->groupsA = 1;
     if (tcfir) {
         p->kernelA = tcfir;
         p->formA = "tensor-int8";
@@ -1547,8 +1563,7 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
         ca.s0 = s0;
         ca.sc = sc;
         void *argsA[] = {&ca};
-        int ga = (int)std::min<long long>(nA, (long long)ca.tiles * sc);
-        ga = std::max(ca.G, ga / ca.G * ca.G);
+        const int ga = grid_a(nA, p->groupsA, ca.G, (long long)ca.tiles * sc);
         vspec_status r = launch(p, 0, sc * nsub, p->kernelA, dim3(ga), dim3(p->TA), argsA, p->smemA, st);
         if (r != VSPEC_OK) return r;
         cb.s0 = s0;
@@ -1751,8 +1766,7 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
             ca.sc = sc;
             void *argsA[] = {&ca};
             // no more CTAs than items, and a whole number of tile groups
-            int ga = (int)std::min<long long>(nA, (long long)ca.tiles * sc);
-            ga = std::max(ca.G, ga / ca.G * ca.G);
+            const int ga = grid_a(nA, p->groupsA, ca.G, (long long)ca.tiles * sc);
             vspec_status r = launch(p, 0, sc, p->kernelA, dim3(ga), dim3(p->TA), argsA, p->smemA, st);
             if (r != VSPEC_OK) return r;
         }
@@ -2143,6 +2157,11 @@ vspec_status vspec_debug_flags(unsigned *flags, int clear) {
     VSPEC_CUDA(vspec_bp_debug_flags(&bp_flags, clear != 0));
     VSPEC_CUDA(vspec_rowbatch_debug_flags(&row_flags, clear != 0));
     *flags |= ring_flags | bp_flags | row_flags;
+    for (auto fn : {vspec_colgrp8_debug_flags}) {
+        unsigned f = 0;
+        VSPEC_CUDA(fn(&f, clear != 0));
+        *flags |= f;
+    }
     return VSPEC_OK;
 #else
     (void)flags;

@@ -93,6 +93,9 @@ struct ColParams {
     // interleaved rows instead, word w being column w / nsub of band w mod nsub
     int nsub = 1, band = 0, lsub = 0;
     long long zstride = 0;  // scratch elements per spectrum (0: N)
+    // single-pol pairs (fir_colgrp_kernel, fir_coldir_kernel): pair s holds the
+    // chunk's spectra s and s + half, of which spectra below nreal exist
+    int half = 0, nreal = 0;
 };
 
 struct RowParams {
@@ -466,7 +469,9 @@ __global__ void __launch_bounds__(512) fir_colfft_kernel(const __grid_constant__
 
 // Kernel A, register-column form: dual-pol PFB of at most 8 taps in tiles of
 // 512 points (one per thread) with columns of N2 = 2 .. 128 points (nchan
-// 2^12 .. 2^18 with 2048-point rows, 2^19 with 4096-point rows). The FIR
+// 2^12 .. 2^18 with 2048-point rows, 2^19 with 4096-point rows). Plans launch it
+// for columns of at most 16 points (longer ones: vspec_colgrp.cuh); the
+// persistent forms run its tile body at every length. The FIR
 // stage is the same register
 // window as above. Columns of at most 16 points (R1 == N2) are then whole
 // length-N2 DFTs in registers, one column per thread, in natural output

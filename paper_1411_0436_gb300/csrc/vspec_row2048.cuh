@@ -38,6 +38,7 @@
 #include "vspec_kernels.cuh"
 #include "vspec_kernels_tc.cuh"
 #include "vspec_tc.cuh"
+#include "vspec_tmem.cuh"
 
 namespace vspec {
 
@@ -50,53 +51,6 @@ struct Row2048 {
     static constexpr size_t smem = (size_t)NBUF * ROW_BYTES + TW2 * 8 + NBUF * 12 + 8;
     static_assert(smem <= 232448, "shared memory of one CTA");
 };
-
-__device__ __forceinline__ void tmem_ld32_async(uint32_t taddr, uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x32.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31}, [%32];"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]),
-          "=r"(r[15]), "=r"(r[16]), "=r"(r[17]), "=r"(r[18]), "=r"(r[19]), "=r"(r[20]), "=r"(r[21]),
-          "=r"(r[22]), "=r"(r[23]), "=r"(r[24]), "=r"(r[25]), "=r"(r[26]), "=r"(r[27]), "=r"(r[28]),
-          "=r"(r[29]), "=r"(r[30]), "=r"(r[31])
-        : "r"(taddr) : "memory");
-}
-// The wait carries the loaded registers, so that no use of them is scheduled before it.
-__device__ __forceinline__ void tmem_ld32_wait(uint32_t (&r)[32]) {
-    asm volatile("tcgen05.wait::ld.sync.aligned;"
-                 : "+r"(r[0]), "+r"(r[1]), "+r"(r[2]), "+r"(r[3]), "+r"(r[4]), "+r"(r[5]), "+r"(r[6]), "+r"(r[7]),
-                   "+r"(r[8]), "+r"(r[9]), "+r"(r[10]), "+r"(r[11]), "+r"(r[12]), "+r"(r[13]), "+r"(r[14]),
-                   "+r"(r[15]), "+r"(r[16]), "+r"(r[17]), "+r"(r[18]), "+r"(r[19]), "+r"(r[20]), "+r"(r[21]),
-                   "+r"(r[22]), "+r"(r[23]), "+r"(r[24]), "+r"(r[25]), "+r"(r[26]), "+r"(r[27]), "+r"(r[28]),
-                   "+r"(r[29]), "+r"(r[30]), "+r"(r[31])
-                 :: "memory");
-}
-__device__ __forceinline__ void tmem_st32(uint32_t taddr, const uint32_t (&r)[32]) {
-    asm volatile(
-        "tcgen05.st.sync.aligned.32x32b.x32.b32 [%32], "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15, "
-        "%16, %17, %18, %19, %20, %21, %22, %23, %24, %25, %26, %27, %28, %29, %30, %31};"
-        :: "r"(r[0]), "r"(r[1]), "r"(r[2]), "r"(r[3]), "r"(r[4]), "r"(r[5]), "r"(r[6]), "r"(r[7]), "r"(r[8]),
-           "r"(r[9]), "r"(r[10]), "r"(r[11]), "r"(r[12]), "r"(r[13]), "r"(r[14]), "r"(r[15]), "r"(r[16]),
-           "r"(r[17]), "r"(r[18]), "r"(r[19]), "r"(r[20]), "r"(r[21]), "r"(r[22]), "r"(r[23]), "r"(r[24]),
-           "r"(r[25]), "r"(r[26]), "r"(r[27]), "r"(r[28]), "r"(r[29]), "r"(r[30]), "r"(r[31]), "r"(taddr)
-        : "memory");
-}
-
-__device__ __forceinline__ void tmem_ld16_wait(uint32_t taddr, float (&v)[16]) {
-    uint32_t r[16];
-    asm volatile(
-        "tcgen05.ld.sync.aligned.32x32b.x16.b32 "
-        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];\n\t"
-        "tcgen05.wait::ld.sync.aligned;"
-        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]),
-          "=r"(r[8]), "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
-        : "r"(taddr) : "memory");
-#pragma unroll
-    for (int i = 0; i < 16; i++) v[i] = __uint_as_float(r[i]);
-}
 
 // Order of a 16-point butterfly's loads: the inputs of its first additions
 // (0 and 8, 4 and 12, ...) arrive next to each other.
@@ -230,7 +184,7 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
             for (int k = 0; k < 2; k++) {
                 uint32_t a[32];
                 if (run) {
-                    tmem_ld32_async(tm_run + 32 * k, a);
+                    tmem_ld<32>(tm_run + 32 * k, a);
                 } else {
 #pragma unroll
                     for (int e = 0; e < 32; e++) a[e] = 0u;
@@ -246,7 +200,7 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
                     __syncwarp();
                 }
                 Dft<8>::run(v);
-                if (run) tmem_ld32_wait(a);
+                if (run) tmem_wait<32>(a);
 #pragma unroll
                 for (int q = 0; q < 8; q++) {
                     float4 c = make_float4(__uint_as_float(a[4 * q]), __uint_as_float(a[4 * q + 1]),
@@ -262,8 +216,8 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
                 } else {
                     if (totals) {
                         uint32_t t[32];
-                        tmem_ld32_async(tm_tot + 32 * k, t);
-                        tmem_ld32_wait(t);
+                        tmem_ld<32>(tm_tot + 32 * k, t);
+                        tmem_wait<32>(t);
 #pragma unroll
                         for (int e = 0; e < 32; e++)
                             a[e] = __float_as_uint(__uint_as_float(t[e]) + __uint_as_float(a[e]));

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             uint32_t a[32];
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");  // the previous batch's sums
             if (!fresh) {
-                tmem_ld32_async(tm, a);
+                tmem_ld<32>(tm, a);
             } else {
 #pragma unroll
                 for (int e = 0; e < 32; e++) a[e] = 0u;
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
                     for (int q = 0; q < 8; q++) v[q] = d[q ^ (b8 & 7)];
                     Dft<8>::run(v);
                 }
-                if (i == 0 && !fresh) tmem_ld32_wait(a);  // (a warp's lanes share sb: N / 8 is a multiple of 32)
+                if (i == 0 && !fresh) tmem_wait<32>(a);  // (a warp's lanes share sb: N / 8 is a multiple of 32)
                 if (sb < pairs) {
 #pragma unroll
                     for (int q = 0; q < 8; q++) {
@@ -267,8 +267,8 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             if constexpr (NPOL == 2) {
                 uint32_t a[32];
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                tmem_ld32_async(tm, a);
-                tmem_ld32_wait(a);
+                tmem_ld<32>(tm, a);
+                tmem_wait<32>(a);
 #pragma unroll
                 for (int q = 0; q < 8; q++)
                     red[set * N + 8 * b8 + (q ^ (b8 & 7))] =
