@@ -197,10 +197,9 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
         for (int s = s_beg; s < s_end; s += SPB) {
             const int nb = min(SPB, s_end - s);
             uint32_t cf[32];
-            tmem_ld<(G::NCF + 7) / 8 * 8>(tm, cf);
+            tmem_ld_wait<(G::NCF + 7) / 8 * 8>(tm, cf);
             asm volatile("cp.async.wait_group 0;" ::: "memory");
             bar();  // the batch's frames are visible; data is free
-            tmem_wait<(G::NCF + 7) / 8 * 8>(cf);
 #pragma unroll
             for (int k = 0; k < KP; k++) {
                 const int pt = t + TG * k;
@@ -253,8 +252,7 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                 return make_float2(__uint_as_float(tw[2 * i]), __uint_as_float(tw[2 * i + 1]));
             };
             if constexpr (G::kOnePass) {
-                tmem_ld<NTW>(tm + 32, tw);
-                tmem_wait<NTW>(tw);
+                tmem_ld_wait<NTW>(tm + 32, tw);
 #pragma unroll
                 for (int k = 0; k < SPB * C / TG; k++) {
                     const int e = t + TG * k, c = e % C, sb = e / C;
@@ -286,9 +284,8 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                         for (int q = 1; q < R1; q++) d[G::pad(q * M1 * C)] = cmul(v[q], twc[M1 * (q - 1) + j]);
                     }
                 }
-                tmem_ld<NTW>(tm + 32, tw);
+                tmem_ld_wait<NTW>(tm + 32, tw);
                 bar();
-                tmem_wait<NTW>(tw);
                 // second pass: block b of column (sb, c), rows b R2 + q, to the scratch
 #pragma unroll
                 for (int k = 0; k < SPB * C * R1 / TG; k++) {

@@ -182,13 +182,6 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");  // the previous spectrum's sums
 #pragma unroll
             for (int k = 0; k < 2; k++) {
-                uint32_t a[32];
-                if (run) {
-                    tmem_ld<32>(tm_run + 32 * k, a);
-                } else {
-#pragma unroll
-                    for (int e = 0; e < 32; e++) a[e] = 0u;
-                }
                 P2 v[8];
                 const P2 *r3 = row + 8 * (ht + 128 * k);
 #pragma unroll
@@ -199,8 +192,14 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
                     if (ht == 0 && i + G::NBUF < n && !*gave_up) issue(i + G::NBUF);
                     __syncwarp();
                 }
+                uint32_t a[32];
+                if (run) {
+                    tmem_ld_wait<32>(tm_run + 32 * k, a);
+                } else {
+#pragma unroll
+                    for (int e = 0; e < 32; e++) a[e] = 0u;
+                }
                 Dft<8>::run(v);
-                if (run) tmem_wait<32>(a);
 #pragma unroll
                 for (int q = 0; q < 8; q++) {
                     float4 c = make_float4(__uint_as_float(a[4 * q]), __uint_as_float(a[4 * q + 1]),
@@ -216,8 +215,7 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
                 } else {
                     if (totals) {
                         uint32_t t[32];
-                        tmem_ld<32>(tm_tot + 32 * k, t);
-                        tmem_wait<32>(t);
+                        tmem_ld_wait<32>(tm_tot + 32 * k, t);
 #pragma unroll
                         for (int e = 0; e < 32; e++)
                             a[e] = __float_as_uint(__uint_as_float(t[e]) + __uint_as_float(a[e]));

@@ -211,7 +211,7 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             uint32_t a[32];
             asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");  // the previous batch's sums
             if (!fresh) {
-                tmem_ld<32>(tm, a);
+                tmem_ld_wait<32>(tm, a);
             } else {
 #pragma unroll
                 for (int e = 0; e < 32; e++) a[e] = 0u;
@@ -219,15 +219,12 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
 #pragma unroll
             for (int i = 0; i < 2; i++) {
                 const int sb = set + G::SETS * i;
-                P2 v[8];
                 if (sb < pairs) {
                     const P2 *d = data + sb * N + 8 * b8;
+                    P2 v[8];
 #pragma unroll
                     for (int q = 0; q < 8; q++) v[q] = d[q ^ (b8 & 7)];
                     Dft<8>::run(v);
-                }
-                if (i == 0 && !fresh) tmem_wait<32>(a);  // (a warp's lanes share sb: N / 8 is a multiple of 32)
-                if (sb < pairs) {
 #pragma unroll
                     for (int q = 0; q < 8; q++) {
                         float4 c = make_float4(__uint_as_float(a[4 * q]), __uint_as_float(a[4 * q + 1]),
@@ -267,8 +264,7 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             if constexpr (NPOL == 2) {
                 uint32_t a[32];
                 asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-                tmem_ld<32>(tm, a);
-                tmem_wait<32>(a);
+                tmem_ld_wait<32>(tm, a);
 #pragma unroll
                 for (int q = 0; q < 8; q++)
                     red[set * N + 8 * b8 + (q ^ (b8 & 7))] =
