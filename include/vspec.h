@@ -151,8 +151,8 @@ VSPEC_API vspec_status vspec_plan_get_shape(const vspec_plan *plan, int *col_len
  *   input   int8 [(nspectra + P_eff - 1) * nchan][nsub][npol][re, im]
  *           (the sub-bands of one time sample are adjacent);
  *   output  [nsub][nchan] of float4 (npol == 2) or float (npol == 1).
- * Dual-pol plans whose kernel A is a register-column form (PFB of 5..8 taps
- * or direct mode with 2048-point rows; a fused plan's own two-kernel plan
+ * Dual-pol plans whose kernel A is a register-column form (PFB or direct mode
+ * with 2048-point rows; a fused plan's own two-kernel plan
  * counts) read each sub-band of the input in place: every sub-band of a chunk
  * runs in one kernel-A and one kernel-B launch, so the input is read from HBM
  * once (sub-band after sub-band over chunks of about 32 MiB of input where a
@@ -325,8 +325,9 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  *                            two-kernel plan it switches to
  *   two-kernel               the general path
  *   A=colreg|coldir|general|gather|none   kernel A's form: register columns
- *                            (dual-pol PFB), register columns (dual-pol
- *                            direct), the general kernel, taps read from the
+ *                            (dual-pol PFB; colreg4, colreg16: up to 4, up to
+ *                            16 taps), register columns (dual-pol direct), the
+ *                            general kernel, taps read from the
  *                            input (gather-blocked: from frames staged in
  *                            shared memory); none for one-row transforms
  *   B=row2048|general|tensor kernel B's form (-batched: the one-row kernel of

@@ -36,9 +36,13 @@ using vspec::Pass;
 // vspec_ring.cu
 const void *vspec_pick_kernel_ring(int N2, size_t *smem);
 cudaError_t vspec_ring_debug_flags(unsigned *flags, bool clear);
-// vspec_colgrp8.cu
-const void *vspec_pick_kernel_colgrp8(int N2, size_t *smem, int *groups);
+// vspec_colgrp4.cu, vspec_colgrp8.cu, vspec_colgrp16.cu
+const void *vspec_pick_kernel_colgrp4(int N2, int npol, size_t *smem, int *groups);
+const void *vspec_pick_kernel_colgrp8(int N2, int npol, size_t *smem, int *groups);
+const void *vspec_pick_kernel_colgrp16(int N2, int npol, size_t *smem, int *groups);
+cudaError_t vspec_colgrp4_debug_flags(unsigned *flags, bool clear);
 cudaError_t vspec_colgrp8_debug_flags(unsigned *flags, bool clear);
+cudaError_t vspec_colgrp16_debug_flags(unsigned *flags, bool clear);
 // vspec_rowbatch.cu
 const void *vspec_pick_kernel_rowbatch(int nchan, int npol, int P, size_t *smem);
 const void *vspec_pick_fold_row(int npol);
@@ -328,8 +332,22 @@ const void *pick_kernel_colreg(int N2, size_t *smem, int *groups, std::vector<in
         case 8: *smem = ColReg<8>::smem; return (const void *)fir_colreg_kernel<8>;
         case 16: *smem = ColReg<16>::smem; return (const void *)fir_colreg_kernel<16>;
     }
-    return vspec_pick_kernel_colgrp8(N2, smem, groups);
+    return vspec_pick_kernel_colgrp8(N2, 2, smem, groups);
 }
+
+// ... for other tap counts (PT: taps rounded up to 4, 8 or 16) and for single
+// polarisation. Kernel A, GB300, general kernel against groups, us: 4 taps
+// 16384 channels (2048 spectra) 164 / 114, 65536 (512) 224 / 135, 262144 (128)
+// 228 / 203; 12 taps 4096 (4096) 91 / 89, 16384 (2048) 217 / 167, 65536 (512)
+// 263 / 210, 524288 (64, gather kernel) 721 / 311; single-pol 8 taps 4096
+// (4096) 55 / 43, 16384 (2048) 99 / 77, 65536 (1024) 244 / 172.
+const void *pick_kernel_colgrp(int N2, int PT, int npol, size_t *smem, int *groups, std::vector<int> *radices) {
+    *radices = N2 <= 16 ? std::vector<int>{N2} : std::vector<int>{8, N2 / 8};
+    return PT == 4 ? vspec_pick_kernel_colgrp4(N2, npol, smem, groups)
+         : PT == 8 ? vspec_pick_kernel_colgrp8(N2, npol, smem, groups)
+                   : vspec_pick_kernel_colgrp16(N2, npol, smem, groups);
+}
+
 
 // Kernel-A CTAs of a launch of `items` (tile, spectrum) items: at most nA, no
 // more workers (groups) than items, whole tile groups.
@@ -729,6 +747,20 @@ vspec_status build_plan(vspec_plan *p) {
         p->gather = gather;
         if (gather) PT = 1;
     }
+    // pre-filtered plans whose rows come out at 2048 points (4096 at 2^19
+    // dual-pol) with columns of at most 128: kernel A in 512-point tiles
+    bool colgrp = false;
+    if (pfb && p->npol == 2 && !p->req_n2 && !p->req_cols && N > kRowElems &&
+        !(p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)) &&
+        (p->npol == 2 || !(p->flags & VSPEC_PLAN_KAHAN))) {
+        const int n2 = std::min(128, N / kRowElems);
+        if ((N / n2 == kRowElems && (p->npol == 2 || n2 <= 64)) || (p->npol == 2 && N / n2 == 2 * kRowElems)) {
+            colgrp = true;
+            N2 = n2;
+            p->gather = false;
+            PT = p->P <= 4 ? 4 : p->P <= 8 ? 8 : 16;
+        }
+    }
     const int N1 = N / N2;
     if (N1 > 4096) {
         g_last_error = "nchan too large for this mode in this build";
@@ -750,8 +782,8 @@ vspec_status build_plan(vspec_plan *p) {
     // dual-pol PFB (5 .. 8 taps) with 2048-point rows (4096 at 2^19): the
     // register-column kernel A in 512-point tiles (for N2 = 128 rows of 4
     // samples, which the tile groups read a whole line at a time)
-    const bool colreg_tiles = p->npol == 2 && pfb && PT == 8 && !p->gather && (N1 == 2048 || N1 == 4096) && N2 >= 2 &&
-                              N2 <= 128 && !p->req_cols;
+    const bool colreg_tiles = colgrp || (p->npol == 2 && pfb && PT == 8 && !p->gather && (N1 == 2048 || N1 == 4096) &&
+                                         N2 >= 2 && N2 <= 128 && !p->req_cols);
     if (colreg_tiles) C = 512 / N2;
     // dual-pol PFB too long for a register window, 512-point columns (2^20):
     // the blocked kernel A, up to its 8 taps (0.78 against 1.77 ms per 100
@@ -813,10 +845,11 @@ vspec_status build_plan(vspec_plan *p) {
     size_t smem_colreg = 0;
     std::vector<int> r_colreg;
     const void *colreg = p->npol == 2 && pfb && PT == 8 && PPT == 1 && !p->gather && N2 * C == 512 && !p->req_cols
-                             ? pick_kernel_colreg(N2, &smem_colreg, &p->groupsA, &r_colreg) : nullptr;
+                             ? pick_kernel_colreg(N2, &smem_colreg, &p->groupsA, &r_colreg)
+                         : colgrp ? pick_kernel_colgrp(N2, PT, p->npol, &smem_colreg, &p->groupsA, &r_colreg) : nullptr;
     if (colreg) {
         p->kernelA = colreg;
-        p->formA = "colreg";
+        p->formA = PT == 4 ? "colreg4" : PT == 16 ? "colreg16" : "colreg";
     }
     // tensor-core plans with 2048-point rows and N2 = 16, 32, 64:
     //  - VSPEC_PLAN_TENSOR_INT8 (PFB of at most 8 taps, or direct): pre-filter
@@ -1504,7 +1537,7 @@ static vspec_plan *sb_plan(vspec_plan *p) { return p->fused && p->assist ? p->as
 // in place: the dual-pol register-column forms on the plain two-kernel path.
 static bool sb_in_place(const vspec_plan *p, int nsub) {
     return nsub > 1 && p->npol == 2 && !p->fused && !p->ring && !p->tc && !p->tc_cols && !p->fir_b && !p->kahan &&
-           (std::strcmp(p->formA, "colreg") == 0 || std::strcmp(p->formA, "coldir") == 0);
+           (std::strncmp(p->formA, "colreg", 6) == 0 || std::strcmp(p->formA, "coldir") == 0);
 }
 
 static void make_params(const vspec_plan *p, const int8_t *d_in, int nspectra, vspec::ColParams &ca,
@@ -2157,7 +2190,7 @@ vspec_status vspec_debug_flags(unsigned *flags, int clear) {
     VSPEC_CUDA(vspec_bp_debug_flags(&bp_flags, clear != 0));
     VSPEC_CUDA(vspec_rowbatch_debug_flags(&row_flags, clear != 0));
     *flags |= ring_flags | bp_flags | row_flags;
-    for (auto fn : {vspec_colgrp8_debug_flags}) {
+    for (auto fn : {vspec_colgrp4_debug_flags, vspec_colgrp8_debug_flags, vspec_colgrp16_debug_flags}) {
         unsigned f = 0;
         VSPEC_CUDA(fn(&f, clear != 0));
         *flags |= f;

@@ -5,15 +5,33 @@
 
 namespace vspec {
 
-// Kernel A for columns of N2 points and PT taps at most, its dynamic shared
-// memory and groups per CTA. Four groups beat two (N2 = 64: 1199 against 1289
+// Groups per CTA. Up to 8 taps four groups beat two (N2 = 64: 1199 against 1289
 // us per 2048 spectra of 131072 channels), although a batch of 4 spectra unpacks
-// 11 frames for 4 outputs and one of 8 spectra 15 for 8.
-template <int N2, int PT> const void *colgrp_instance(size_t *smem, int *groups) {
-    constexpr int GR = 4;
+// 11 frames for 4 outputs and one of 8 spectra 15 for 8. With 16 taps the ring
+// leaves room for two groups, or one beside the 128-point columns' padded tiles.
+template <int N2, int PT> constexpr int colgrp_groups() {
+    return PT <= 8 ? 4 : ColGrp<N2, PT, 2>::smem <= 232448 ? 2 : 1;
+}
+
+// Kernel A for columns of N2 points (2 .. 128) and PT taps at most, its dynamic
+// shared memory and groups per CTA.
+template <int N2, int PT> const void *colgrp_instance(int npol, size_t *smem, int *groups) {
+    constexpr int GR = colgrp_groups<N2, PT>();
     *smem = ColGrp<N2, PT, GR>::smem;
     *groups = GR;
-    return (const void *)fir_colgrp_kernel<N2, PT, GR, 2>;
+    return npol == 2 ? (const void *)fir_colgrp_kernel<N2, PT, GR, 2> : (const void *)fir_colgrp_kernel<N2, PT, GR, 1>;
+}
+template <int PT> const void *pick_colgrp(int N2, int npol, size_t *smem, int *groups) {
+    switch (N2) {
+        case 2: return colgrp_instance<2, PT>(npol, smem, groups);
+        case 4: return colgrp_instance<4, PT>(npol, smem, groups);
+        case 8: return colgrp_instance<8, PT>(npol, smem, groups);
+        case 16: return colgrp_instance<16, PT>(npol, smem, groups);
+        case 32: return colgrp_instance<32, PT>(npol, smem, groups);
+        case 64: return colgrp_instance<64, PT>(npol, smem, groups);
+        case 128: return colgrp_instance<128, PT>(npol, smem, groups);
+    }
+    return nullptr;
 }
 
 // This translation unit's bounds-check status word (debug builds).
