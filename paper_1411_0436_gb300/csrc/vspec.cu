@@ -43,6 +43,9 @@ const void *vspec_pick_kernel_colgrp16(int N2, int npol, size_t *smem, int *grou
 cudaError_t vspec_colgrp4_debug_flags(unsigned *flags, bool clear);
 cudaError_t vspec_colgrp8_debug_flags(unsigned *flags, bool clear);
 cudaError_t vspec_colgrp16_debug_flags(unsigned *flags, bool clear);
+// vspec_coldirgrp.cu
+const void *vspec_pick_kernel_coldirgrp(int N2, int npol, size_t *smem, int *groups);
+cudaError_t vspec_coldirgrp_debug_flags(unsigned *flags, bool clear);
 // vspec_rowbatch.cu
 const void *vspec_pick_kernel_rowbatch(int nchan, int npol, int P, size_t *smem);
 const void *vspec_pick_fold_row(int npol);
@@ -198,6 +201,7 @@ struct vspec_plan {
     int *tc_status = nullptr;  // bounded-wait flag of the tensor-core or ring kernel
     int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel (in twB's allocation)
     float2 *twBt = nullptr;      // its twiddles (in twB's allocation)
+    bool pair = false;           // single-pol plans whose kernels run two spectra at once (scratch elements are pairs)
     int groupsA = 1;             // independent groups per kernel-A CTA (fir_colgrp_kernel)
     bool row_groups = false;     // kernel B is row2048_group_kernel
     bool row_batch = false;      // kernel B is row_batch_kernel (one-row transforms)
@@ -267,22 +271,15 @@ template <int NPOL> const void *pick_kernel_a(int PT, int PPT) {
     return nullptr;
 }
 
-// register-column kernel A for dual-pol direct FFT (2048-point tiles), N2 in
-// 2 .. 256, and its column pass list (one pass up to 16 points, then 16 x N2/16)
-const void *pick_kernel_coldir(int N2, size_t *smem, std::vector<int> *radices) {
-    using namespace vspec;
+// kernel A for direct FFT with 2048-point rows (2048-point tiles), N2 in
+// 2 .. 256, and its column pass list (one pass up to 16 points, then 16 x N2/16).
+// GB300, us, one 512-thread group per CTA against four of 128: N2 = 2 (4096
+// spectra) 61 / 57, 16 (512) 63 / 61, 64 (256) 134 / 119, 256 (256) 626 / 518;
+// single-pol, general kernel against pairs: 2 (4096) 51 / 30, 32 (512) 123 / 63,
+// 256 (64) 152 / 95.
+const void *pick_kernel_coldir(int N2, int npol, size_t *smem, int *groups, std::vector<int> *radices) {
     *radices = N2 <= 16 ? std::vector<int>{N2} : std::vector<int>{16, N2 / 16};
-    switch (N2) {
-        case 2: *smem = ColDir<2>::smem; return (const void *)fir_coldir_kernel<2>;
-        case 4: *smem = ColDir<4>::smem; return (const void *)fir_coldir_kernel<4>;
-        case 8: *smem = ColDir<8>::smem; return (const void *)fir_coldir_kernel<8>;
-        case 16: *smem = ColDir<16>::smem; return (const void *)fir_coldir_kernel<16>;
-        case 32: *smem = ColDir<32>::smem; return (const void *)fir_coldir_kernel<32>;
-        case 64: *smem = ColDir<64>::smem; return (const void *)fir_coldir_kernel<64>;
-        case 128: *smem = ColDir<128>::smem; return (const void *)fir_coldir_kernel<128>;
-        case 256: *smem = ColDir<256>::smem; return (const void *)fir_coldir_kernel<256>;
-    }
-    return nullptr;
+    return vspec_pick_kernel_coldirgrp(N2, npol, smem, groups);
 }
 
 // kernel A with the column DFTs on the tensor cores (dual-pol PFB, 8 taps,
@@ -347,7 +344,6 @@ const void *pick_kernel_colgrp(int N2, int PT, int npol, size_t *smem, int *grou
          : PT == 8 ? vspec_pick_kernel_colgrp8(N2, npol, smem, groups)
                    : vspec_pick_kernel_colgrp16(N2, npol, smem, groups);
 }
-
 
 // Kernel-A CTAs of a launch of `items` (tile, spectrum) items: at most nA, no
 // more workers (groups) than items, whole tile groups.
@@ -582,6 +578,11 @@ constexpr int kRingSlotsPerLaunch = 4096;
 // so that the bands after the first find it in L2.
 constexpr size_t kSbInPlaceBytes = 32u << 20;
 
+// Chunk scratch of `spectra` spectra (pairs: an odd count takes a whole last pair).
+size_t z_bytes(const vspec_plan *p, int spectra) {
+    return (size_t)(p->pair ? spectra + (spectra & 1) : spectra) * p->N * (p->npol == 2 ? sizeof(float4) : sizeof(float2));
+}
+
 // Partial-sum slots a kernel-B launch of n CTAs uses: a CTA's rank among the
 // CTAs that share a row tile stays below n / tiles + 2 (span_slot).
 int slots_for(const vspec_plan *p, int n) { return n / (p->N2 / p->RB) + 2; }
@@ -748,7 +749,9 @@ vspec_status build_plan(vspec_plan *p) {
         if (gather) PT = 1;
     }
     // pre-filtered plans whose rows come out at 2048 points (4096 at 2^19
-    // dual-pol) with columns of at most 128: kernel A in 512-point tiles
+    // dual-pol) with columns of at most 128 (single-pol 64: 128-point columns
+    // would make 8-byte tile rows, 292 us per 128 spectra of 262144 channels
+    // against 287 on 4096-point rows): kernel A in 512-point tiles
     bool colgrp = false;
     if (pfb && p->npol == 2 && !p->req_n2 && !p->req_cols && N > kRowElems &&
         !(p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)) &&
@@ -772,12 +775,12 @@ vspec_status build_plan(vspec_plan *p) {
     const int pts_target = PT == 1 ? 4096 : 512;
     int C = std::max(cmin, pts_target / N2);
     C = std::min(C, N1);
-    // dual-pol direct FFT with 2048-point rows: the register-column kernel A
-    // in tiles of 2048 points
+    // direct FFT with 2048-point rows: kernel A in tiles of 2048 points
     size_t smem_coldir = 0;
     std::vector<int> r_coldir;
-    const void *coldir = p->npol == 2 && !pfb && N1 == 2048 && N2 >= 2 && N2 <= 256 && !p->req_cols
-                             ? pick_kernel_coldir(N2, &smem_coldir, &r_coldir) : nullptr;
+    const void *coldir = p->npol == 2 && !pfb && N1 == 2048 && N2 >= 2 && N2 <= 256 && !p->req_cols &&
+                                 (p->npol == 2 || !(p->req_n2 || (p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR))))
+                             ? pick_kernel_coldir(N2, p->npol, &smem_coldir, &p->groupsA, &r_coldir) : nullptr;
     if (coldir) C = 2048 / N2;
     // dual-pol PFB (5 .. 8 taps) with 2048-point rows (4096 at 2^19): the
     // register-column kernel A in 512-point tiles (for N2 = 128 rows of 4
@@ -813,9 +816,11 @@ vspec_status build_plan(vspec_plan *p) {
     p->TA = TA;
     p->kernelA = p->gather ? (p->npol == 2 ? pick_kernel_gather<2>(PPT) : pick_kernel_gather<1>(PPT))
                            : (p->npol == 2 ? pick_kernel_a<2>(PT, PPT) : pick_kernel_a<1>(PT, PPT));
+    // single polarisation in these forms: two spectra per scratch element
+    p->pair = p->npol == 1 && (coldir || colgrp);
     if (coldir) {
         p->kernelA = coldir;
-        p->formA = "coldir";
+        p->formA = p->pair ? "general-paired" : "coldir";
     }
     if (p->gather) p->formA = "gather";
     if (colblk) {
@@ -849,7 +854,7 @@ vspec_status build_plan(vspec_plan *p) {
                          : colgrp ? pick_kernel_colgrp(N2, PT, p->npol, &smem_colreg, &p->groupsA, &r_colreg) : nullptr;
     if (colreg) {
         p->kernelA = colreg;
-        p->formA = PT == 4 ? "colreg4" : PT == 16 ? "colreg16" : "colreg";
+        p->formA = p->pair ? "general-paired" : PT == 4 ? "colreg4" : PT == 16 ? "colreg16" : "colreg";
     }
     // tensor-core plans with 2048-point rows and N2 = 16, 32, 64:
     //  - VSPEC_PLAN_TENSOR_INT8 (PFB of at most 8 taps, or direct): pre-filter
@@ -948,9 +953,10 @@ vspec_status build_plan(vspec_plan *p) {
         p->passB[1].r == 16 && p->passB[2].r == 8) {
         using namespace vspec;
         const bool k = p->kahan, f = p->fir_b;
-        p->row_groups = p->npol == 2 && !k && !f;
+        p->row_groups = (p->npol == 2 && !k && !f) || p->pair;
         if (p->row_groups)  // coltc: scratch elements in the tensor-core column kernel's order
-            p->kernelB = coltc ? (const void *)row2048_group_kernel<true> : (const void *)row2048_group_kernel<false>;
+            p->kernelB = p->pair ? (const void *)row2048_group_kernel<kRowPairs>
+                         : coltc ? (const void *)row2048_group_kernel<kRowSplit> : (const void *)row2048_group_kernel<kRowPacked>;
         else if (p->npol == 2 && coltc)
             p->kernelB = (const void *)row2048_kernel<2, true, false, true>;
         else if (p->npol == 2)
@@ -969,8 +975,13 @@ vspec_status build_plan(vspec_plan *p) {
     // kernel; compensated plans, and dual-pol 2048 channels with more than 8
     // taps, keep the kernels above)
     const void *kernelB_limits = p->kernelB;  // the kernel whose occupancy sets the launch limits
-    const int TB_limits = p->TB;
-    const size_t smem_limits = p->smemB;
+    int TB_limits = p->TB;
+    size_t smem_limits = p->smemB;
+    if (p->pair) {
+        kernelB_limits = (const void *)vspec::row2048_kernel<1, false, false>;
+        TB_limits = 256;
+        smem_limits = 2 * (size_t)vspec::kRow2048Stride * elem;
+    }
     if (p->fir_b && !p->kahan) {
         size_t smem = 0;
         if (const void *k = vspec_pick_kernel_rowbatch(N, p->npol, p->P, &smem)) {
@@ -1035,7 +1046,7 @@ vspec_status build_plan(vspec_plan *p) {
     // (row2048_group_kernel and row_batch_kernel run one CTA per SM, but keep
     // the limits of the kernels that run the other plans of their sizes)
     p->maxB = p->row_groups ? std::max(2, p->occB) : p->occB;
-    if (p->row_batch) {
+    if (p->row_batch || p->pair) {
         VSPEC_CUDA(raise_smem_cap(kernelB_limits, smem_limits));
         VSPEC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->maxB, kernelB_limits, TB_limits, smem_limits));
         p->maxB = std::max(p->maxB, p->occB);
@@ -1069,7 +1080,7 @@ vspec_status build_plan(vspec_plan *p) {
         if ((st = dev_alloc((void **)&p->ring_ctl, sizeof(int) * (2 + 2 * (size_t)kRingSlotsPerLaunch), &tot)))
             return st;
     }
-    if ((st = dev_alloc(&p->Z, (size_t)std::max(1, p->sc_alloc) * N * elem, &tot))) return st;
+    if ((st = dev_alloc(&p->Z, z_bytes(p, std::max(1, p->sc_alloc)), &tot))) return st;
     if ((st = dev_alloc(&p->partial, (size_t)p->slots_cap * N * accel, &tot))) return st;
     if (p->tc || p->tc_cols || p->ring) {
         if ((st = dev_alloc((void **)&p->tc_status, sizeof(int), &tot))) return st;
@@ -1418,12 +1429,11 @@ vspec_status vspec_plan_set_tuning(vspec_plan *plan, const vspec_tuning *t) {
     }
     if (tk) {
         if (!tk->fir_b && t->chunk_spectra > tk->sc_alloc) {  // grow the chunk scratch
-            const size_t elem = tk->npol == 2 ? sizeof(float4) : sizeof(float2);
-            const size_t old_bytes = (size_t)tk->sc_alloc * tk->N * elem;
+            const size_t old_bytes = z_bytes(tk, tk->sc_alloc);
             void *z = nullptr;
             size_t tot = 0;
             VSPEC_CUDA(cudaDeviceSynchronize());
-            vspec_status st = dev_alloc(&z, (size_t)t->chunk_spectra * tk->N * elem, &tot);
+            vspec_status st = dev_alloc(&z, z_bytes(tk, t->chunk_spectra), &tot);
             if (st != VSPEC_OK) return st;
             cudaFree(tk->Z);
             tk->Z = z;
@@ -1505,13 +1515,12 @@ vspec_status vspec_plan_trim_scratch(vspec_plan *plan) {
     if (!plan) return VSPEC_ERR_INVALID_ARG;
     vspec_plan *tk = plan->fused ? plan->assist : plan;
     if (!tk || tk->fir_b || tk->sc_alloc <= tk->sc_max) return VSPEC_OK;
-    const size_t elem = tk->npol == 2 ? sizeof(float4) : sizeof(float2);
-    const size_t old_bytes = (size_t)tk->sc_alloc * tk->N * elem;
+    const size_t old_bytes = z_bytes(tk, tk->sc_alloc);
     VSPEC_CUDA(cudaDeviceSynchronize());
     cudaFree(tk->Z);
     tk->Z = nullptr;
     size_t tot = 0;
-    vspec_status st = dev_alloc(&tk->Z, (size_t)tk->sc_max * tk->N * elem, &tot);
+    vspec_status st = dev_alloc(&tk->Z, z_bytes(tk, tk->sc_max), &tot);
     if (st != VSPEC_OK) {
         tk->sc_alloc = 0;
         tk->scratch_bytes -= old_bytes;
@@ -1774,7 +1783,8 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
     const int sc_full = (nspectra + nchunks - 1) / nchunks;
     // slots of the largest kernel-B launch (no more CTAs than items)
     const int tilesB = p->N2 / p->RB;
-    int slots = slots_for(p, (int)std::min<long long>(nB, (long long)tilesB * sc_full));
+    auto rows = [&](int sc) { return p->pair ? (sc + 1) / 2 : sc; };  // scratch spectra of sc spectra
+    int slots = slots_for(p, (int)std::min<long long>(nB, (long long)tilesB * rows(sc_full)));
     // a one-row transform in one launch: block k is the only writer of slot k
     // and stores it, so nothing needs zeroing and the fold reads those slots
     const bool store = p->fir_b && !p->kahan && !p->tc && nchunks == 1;
@@ -1796,19 +1806,21 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
         const int sc = std::min(sc_full, nspectra - s0);
         if (!p->fir_b) {
             ca.s0 = s0;
-            ca.sc = sc;
+            ca.sc = rows(sc);
+            ca.half = rows(sc);
+            ca.nreal = sc;
             void *argsA[] = {&ca};
-            // no more CTAs than items, and a whole number of tile groups
-            const int ga = grid_a(nA, p->groupsA, ca.G, (long long)ca.tiles * sc);
+            // no more workers than items, and a whole number of tile groups
+            const int ga = grid_a(nA, p->groupsA, ca.G, (long long)ca.tiles * rows(sc));
             vspec_status r = launch(p, 0, sc, p->kernelA, dim3(ga), dim3(p->TA), argsA, p->smemA, st);
             if (r != VSPEC_OK) return r;
         }
         vspec_status r;
         cb.s0 = s0;
-        cb.sc = sc;
+        cb.sc = rows(sc);
         vspec::TcStatus ts{p->tc_status, g_wait_limit.load()};
         void *argsB[] = {&cb, &ts};
-        const int gb = (int)std::min<long long>(nB, (long long)cb.tiles * sc);
+        const int gb = (int)std::min<long long>(nB, (long long)cb.tiles * rows(sc));
         // (a 2048-channel plan reports its one-pass kernel as such)
         const int kind = p->owner && p->owner->row_plan == p ? 3 : 1;
         r = launch(p, kind, sc, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st);
@@ -2190,7 +2202,8 @@ vspec_status vspec_debug_flags(unsigned *flags, int clear) {
     VSPEC_CUDA(vspec_bp_debug_flags(&bp_flags, clear != 0));
     VSPEC_CUDA(vspec_rowbatch_debug_flags(&row_flags, clear != 0));
     *flags |= ring_flags | bp_flags | row_flags;
-    for (auto fn : {vspec_colgrp4_debug_flags, vspec_colgrp8_debug_flags, vspec_colgrp16_debug_flags}) {
+    for (auto fn : {vspec_colgrp4_debug_flags, vspec_colgrp8_debug_flags, vspec_colgrp16_debug_flags,
+                    vspec_coldirgrp_debug_flags}) {
         unsigned f = 0;
         VSPEC_CUDA(fn(&f, clear != 0));
         *flags |= f;

@@ -19,6 +19,9 @@ pytestmark = pytest.mark.gpu
     (262144, 3, 2, PFB, WIN_HANN, 2, 0, 0), (65536, 8, 2, PFB, WIN_HANN, 11, 2, 0), (262144, 8, 2, PFB, WIN_HANN, 5, 8, 0),
     (4096, 16, 2, PFB, WIN_HANN, 37, 1, 0), (8192, 9, 2, PFB, WIN_HAMMING, 8, 0, 0), (32768, 12, 2, PFB, WIN_HANN, 19, 2, 7),
     (131072, 16, 2, PFB, WIN_HANN, 9, 4, 0), (262144, 12, 2, PFB, WIN_HANN, 18, 16, 0), (524288, 16, 2, PFB, WIN_HANN, 2, 0, 0),
+    # dual-pol direct
+    (4096, 1, 2, DIRECT, WIN_HANN, 11, 1, 0), (32768, 1, 2, DIRECT, WIN_HAMMING, 6, 2, 0), (65536, 1, 2, DIRECT, WIN_RECT, 9, 1, 4),
+    (524288, 1, 2, DIRECT, WIN_HANN, 5, 8, 0),
 ])
 def test_grouped_kernel_matches_oracle(oracle_mod, n, taps, npol, mode, window, nspectra, blocks_a, chunk):
     from paper_1411_0436_gb300.vspec import PLAN_TWO_KERNEL, Plan
