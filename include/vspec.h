@@ -327,7 +327,8 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  *   A=colreg|coldir|general|gather|none   kernel A's form: register columns
  *                            (dual-pol PFB; colreg4, colreg16: up to 4, up to
  *                            16 taps), register columns (dual-pol direct), the
- *                            general kernel, taps read from the
+ *                            general kernel (general-paired: two single-pol
+ *                            spectra at once), taps read from the
  *                            input (gather-blocked: from frames staged in
  *                            shared memory); none for one-row transforms
  *   B=row2048|general|tensor kernel B's form (-batched: the one-row kernel of

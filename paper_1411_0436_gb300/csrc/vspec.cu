@@ -753,7 +753,7 @@ vspec_status build_plan(vspec_plan *p) {
     // would make 8-byte tile rows, 292 us per 128 spectra of 262144 channels
     // against 287 on 4096-point rows): kernel A in 512-point tiles
     bool colgrp = false;
-    if (pfb && p->npol == 2 && !p->req_n2 && !p->req_cols && N > kRowElems &&
+    if (pfb && !p->req_n2 && !p->req_cols && N > kRowElems &&
         !(p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)) &&
         (p->npol == 2 || !(p->flags & VSPEC_PLAN_KAHAN))) {
         const int n2 = std::min(128, N / kRowElems);
@@ -778,7 +778,7 @@ vspec_status build_plan(vspec_plan *p) {
     // direct FFT with 2048-point rows: kernel A in tiles of 2048 points
     size_t smem_coldir = 0;
     std::vector<int> r_coldir;
-    const void *coldir = p->npol == 2 && !pfb && N1 == 2048 && N2 >= 2 && N2 <= 256 && !p->req_cols &&
+    const void *coldir = !pfb && N1 == 2048 && N2 >= 2 && N2 <= 256 && !p->req_cols &&
                                  (p->npol == 2 || !(p->req_n2 || (p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR))))
                              ? pick_kernel_coldir(N2, p->npol, &smem_coldir, &p->groupsA, &r_coldir) : nullptr;
     if (coldir) C = 2048 / N2;

@@ -19,6 +19,11 @@ pytestmark = pytest.mark.gpu
     (262144, 3, 2, PFB, WIN_HANN, 2, 0, 0), (65536, 8, 2, PFB, WIN_HANN, 11, 2, 0), (262144, 8, 2, PFB, WIN_HANN, 5, 8, 0),
     (4096, 16, 2, PFB, WIN_HANN, 37, 1, 0), (8192, 9, 2, PFB, WIN_HAMMING, 8, 0, 0), (32768, 12, 2, PFB, WIN_HANN, 19, 2, 7),
     (131072, 16, 2, PFB, WIN_HANN, 9, 4, 0), (262144, 12, 2, PFB, WIN_HANN, 18, 16, 0), (524288, 16, 2, PFB, WIN_HANN, 2, 0, 0),
+    # single-pol pre-filter and direct mode: odd and even counts
+    (4096, 8, 1, PFB, WIN_HANN, 1, 0, 0), (8192, 5, 1, PFB, WIN_HANN, 13, 2, 5), (65536, 8, 1, PFB, WIN_HANN, 7, 0, 0),
+    (131072, 2, 1, PFB, WIN_HAMMING, 4, 0, 0), (131072, 8, 1, PFB, WIN_HANN, 5, 16, 0), (16384, 16, 1, PFB, WIN_HANN, 35, 1, 0),
+    (4096, 1, 1, DIRECT, WIN_HANN, 9, 1, 0), (32768, 1, 1, DIRECT, WIN_RECT, 12, 0, 0), (65536, 1, 1, DIRECT, WIN_HAMMING, 5, 2, 3),
+    (524288, 1, 1, DIRECT, WIN_HANN, 3, 0, 0),
     # dual-pol direct
     (4096, 1, 2, DIRECT, WIN_HANN, 11, 1, 0), (32768, 1, 2, DIRECT, WIN_HAMMING, 6, 2, 0), (65536, 1, 2, DIRECT, WIN_RECT, 9, 1, 4),
     (524288, 1, 2, DIRECT, WIN_HANN, 5, 8, 0),
