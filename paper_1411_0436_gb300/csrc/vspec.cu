@@ -161,7 +161,7 @@ struct vspec_plan {
     int sc_alloc = 1;                // chunk spectra the scratch holds now
     int blocks_a = 0, blocks_b = 0;  // CTAs per kernel-A / kernel-B launch, 0: one wave
     bool fir_b = false;              // one-row transform: kernel B only, FIR in its first pass
-    bool fold2048 = false;           // the fold runs reduce2048_kernel (2048-point rows, N2 >= 16)
+    bool fold2048 = false;           // the fold runs reduce2048_kernel or its short form (2048-point rows, N2 >= 2)
     bool gather = false;             // long PFB: kernel A reads the FIR taps from the input
     size_t smemA = 0, smemB = 0;
     std::vector<Pass> passA, passB;
@@ -374,9 +374,10 @@ cudaError_t take_event(vspec_plan *p, cudaEvent_t *ev) {
 }
 
 // Launch one kernel on st (as clusters of `cluster` CTAs if cluster > 1, as a
-// cooperative launch if cluster < 0); in profiling mode bracket it with events.
+// cooperative launch if cluster < 0; pdl: as a dependent of the kernel launched
+// on st just before, see pdl_wait, which the kernel must call); in profiling mode bracket it with events.
 vspec_status launch(vspec_plan *p, int kind, int spectra, const void *fn, dim3 grid, dim3 block,
-                    void **args, size_t smem, cudaStream_t st, int cluster = 0) {
+                    void **args, size_t smem, cudaStream_t st, int cluster = 0, bool pdl = false) {
     vspec_plan *o = p->owner ? p->owner : p;  // an assist plan records into its owner
     vspec_plan::Rec r{kind, spectra, nullptr, nullptr};
     if (o->profiling) {
@@ -416,6 +417,18 @@ vspec_status launch(vspec_plan *p, int kind, int spectra, const void *fn, dim3 g
         cfg.attrs = attr;
         cfg.numAttrs = 1;
         e = cudaLaunchKernelExC(&cfg, fn, args);
+    } else if (pdl && !o->profiling) {  // (profiling: whole kernels between their events)
+        cudaLaunchConfig_t cfg = {};
+        cfg.gridDim = grid;
+        cfg.blockDim = block;
+        cfg.dynamicSmemBytes = smem;
+        cfg.stream = st;
+        cudaLaunchAttribute attr[1];
+        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[0].val.programmaticStreamSerializationAllowed = 1;
+        cfg.attrs = attr;
+        cfg.numAttrs = 1;
+        e = cudaLaunchKernelExC(&cfg, fn, args);
     } else {
         e = cudaLaunchKernel(fn, grid, block, args, smem, st);
     }
@@ -433,10 +446,14 @@ vspec_status launch(vspec_plan *p, int kind, int spectra, const void *fn, dim3 g
     return VSPEC_OK;
 }
 
+constexpr int kFoldSlots = 128;  // above, the fold takes two launches
+
 // Fold `slots` partial-sum slots of p->partial (and p->partial_comp in
 // compensated plans; slots of nsub bands in sub-band calls) into d_accum: with more than 128 slots, first sum each
 // group of 16 slots into its first slot, then fold the group sums.
-vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, cudaStream_t st, int nsub = 1) {
+// (written: the row launch that stored the slots, unless they were zeroed.)
+vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, cudaStream_t st, int nsub = 1,
+                         const vspec::SlotSpan *written = nullptr, bool pdl = false) {
     int groups = slots, stride = nsub;  // a slot holds the nsub bands one after another
     const int N = p->N, N1 = p->N1, N2 = p->N2;
     if (p->row_batch) {
@@ -444,9 +461,9 @@ vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, 
         int n = N, R1 = p->passB[0].r, R2 = p->passB[1].r;
         void *outp = d_accum;
         void *args[] = {&part, &slots, &n, &R1, &R2, &outp};
-        return launch(p, 2, spectra, vspec_pick_fold_row(p->npol), dim3(N / 8), dim3(8, 64), args, 0, st);
+        return launch(p, 2, spectra, vspec_pick_fold_row(p->npol), dim3(N / 8), dim3(8, 64), args, 0, st, 0, pdl);
     }
-    if (slots > 128) {
+    if (slots > kFoldSlots) {
         groups = (slots + 15) / 16;
         stride = 16 * nsub;
         const void *fold = p->npol == 2 ? (p->kahan ? (const void *)vspec::fold_slots_kernel<2, true>
@@ -456,27 +473,38 @@ vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, 
         void *part = p->partial, *pcomp = p->partial_comp;
         int ns = slots, n = N * nsub;
         void *argsF[] = {&part, &pcomp, &ns, &n};
-        vspec_status r = launch(p, 2, 0, fold, dim3((n + 31) / 32, groups), dim3(32, 8), argsF, 0, st);
+        vspec_status r = launch(p, 2, 0, fold, dim3((n + 31) / 32, groups), dim3(32, 8), argsF, 0, st, 0, pdl);
         if (r != VSPEC_OK) return r;
     }
     const void *part = p->partial, *pcomp = p->partial_comp;
     const int *ia = p->invA, *ib = p->invB;
     void *outp = d_accum, *ocomp = p->out_comp;
+    vspec::SlotSpan span = written ? *written : vspec::SlotSpan{0, 1, 1, groups, 0};
     if (p->kahan) {
         void *argsR[] = {&part, &pcomp, &groups, &stride, (void *)&N, (void *)&N1, (void *)&N2, &ia, &ib, &outp, &ocomp};
-        return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32), dim3(32, 8), argsR, 0, st);
+        return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32), dim3(32, 8), argsR, 0, st, 0, pdl);
     }
-    if (p->fold2048) {  // 2048-point rows, N2 >= 16: coalesced through a tile
+    // 2048-point rows: coalesced folds. N2 < 16: the short form where rows are
+    // split over more CTAs than its lanes (N2 = 2, 257 spectra, 78 slots: call
+    // 26.7 -> 23.6 us); with fewer slots its 16 lanes idle (8 bands of 16384
+    // channels, 4 slots: 35 against 53 us) and the channel-order fold is used.
+    if (p->fold2048 && N2 < 16 && groups > 16) {
+        using namespace vspec;
+        const void *k = p->npol == 2 ? (const void *)reduce2048_short_kernel<2> : (const void *)reduce2048_short_kernel<1>;
+        void *argsT[] = {&part, &span, &stride, (void *)&N, (void *)&N2, &ia, &outp};
+        return launch(p, 2, spectra, k, dim3(64 * N2, nsub), dim3(512), argsT, 0, st, 0, pdl);
+    }
+    if (p->fold2048 && N2 >= 16) {
         using namespace vspec;
         // 32 positions per CTA; for N2 < 64 8 positions and 4 slot lanes (more CTAs, shorter chains)
         const bool wide = N2 >= 64;
         const void *k = p->npol == 2 ? (wide ? (const void *)reduce2048_kernel<2, 32, 1> : (const void *)reduce2048_kernel<2, 8, 4>)
                                      : (wide ? (const void *)reduce2048_kernel<1, 32, 1> : (const void *)reduce2048_kernel<1, 8, 4>);
-        void *argsT[] = {&part, &groups, &stride, (void *)&N, (void *)&N2, &ia, &outp};
-        return launch(p, 2, spectra, k, dim3(N2 / 16 * 16 * (wide ? 4 : 16), nsub), dim3(wide ? 256 : 512), argsT, 0, st);
+        void *argsT[] = {&part, &span, &stride, (void *)&N, (void *)&N2, &ia, &outp};
+        return launch(p, 2, spectra, k, dim3(N2 / 16 * 16 * (wide ? 4 : 16), nsub), dim3(wide ? 256 : 512), argsT, 0, st, 0, pdl);
     }
-    void *argsR[] = {&part, &groups, &stride, (void *)&N, (void *)&N1, (void *)&N2, &ia, &ib, &outp};
-    return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32, nsub), dim3(32, 8), argsR, 0, st);
+    void *argsR[] = {&part, &span, &stride, (void *)&N, (void *)&N1, (void *)&N2, &ia, &ib, &outp};
+    return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32, nsub), dim3(32, 8), argsR, 0, st, 0, pdl);
 }
 
 const void *pick_kernel_fused(int logn1, int pt) {
@@ -968,7 +996,7 @@ vspec_status build_plan(vspec_plan *p) {
         p->TB = p->row_groups ? Row2048::THREADS : 256;
         p->smemB = p->row_groups ? Row2048::smem : 2 * (size_t)kRow2048Stride * elem;
         p->formB = "row2048";
-        p->fold2048 = N2 >= 16 && !p->kahan;
+        p->fold2048 = N2 >= 2 && !p->kahan;
     }
     // one-row transforms of 512 .. 2048 channels: the batched one-pass kernel
     // (1024 channels dual-pol, 8 taps, 2048 spectra: 59 us in the general row
@@ -1587,7 +1615,10 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
     const int tilesB = nsub * (p->N2 / p->RB);
     const long long NV = (long long)nsub * p->N;
     const int slots = (int)(std::min<long long>(nB, (long long)tilesB * sc_full) / tilesB + 2);
-    VSPEC_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)slots * NV * sizeof(float4), st));
+    const int gb_full = (int)std::min<long long>(nB, (long long)tilesB * sc_full);
+    const vspec::SlotSpan written{gb_full, tilesB, sc_full, 0, ilog2(p->RB)};
+    const bool store = nchunks == 1 && slots <= kFoldSlots;  // as in run_two_kernel
+    if (!store) VSPEC_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)slots * NV * sizeof(float4), st));
     vspec::ColParams ca;
     vspec::RowParams cb;
     make_params(p, d_in, nspectra, ca, cb);
@@ -1599,7 +1630,7 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
     cb.N = (int)NV;
     cb.tiles = tilesB;
     cb.slots = slots;
-    cb.store = 0;
+    cb.store = store;
     for (int s0 = 0; s0 < nspectra; s0 += sc_full) {
         const int sc = std::min(sc_full, nspectra - s0);
         ca.s0 = s0;
@@ -1613,10 +1644,10 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
         vspec::TcStatus ts{p->tc_status, g_wait_limit.load()};
         void *argsB[] = {&cb, &ts};
         const int gb = (int)std::min<long long>(nB, (long long)tilesB * sc);
-        r = launch(p, 1, sc * nsub, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st);
+        r = launch(p, 1, sc * nsub, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st, 0, p->row_groups);
         if (r != VSPEC_OK) return r;
     }
-    return launch_fold(p, slots, d_accum, nspectra, st, nsub);
+    return launch_fold(p, slots, d_accum, nspectra, st, nsub, store ? &written : nullptr, true);
 }
 
 vspec_status vspec_execute(vspec_plan *plan, const int8_t *d_in, int nspectra, float *d_accum,
@@ -1693,7 +1724,7 @@ static vspec_status run_fused(vspec_plan *p, const int8_t *d_in, int nspectra, f
         vspec_status r = launch(p, 3, nspectra, p->kernelF, dim3(p->cluster * p->nclusters),
                                 dim3(vspec::fusedw::kThreads), argsW, p->smemF, st, p->cluster);
         if (r != VSPEC_OK) return r;
-        return launch_fold(p, p->nclusters, d_accum, nspectra, st);
+        return launch_fold(p, p->nclusters, d_accum, nspectra, st, 1, nullptr, true);
     }
     if (p->fused) {
         vspec::fused::Params fp;
@@ -1712,7 +1743,7 @@ static vspec_status run_fused(vspec_plan *p, const int8_t *d_in, int nspectra, f
         vspec_status r = launch(p, 3, nspectra, p->kernelF, dim3(p->cluster * p->nclusters),
                                 dim3(vspec::fused::kThreads), argsF, p->smemF, st, p->cluster);
         if (r != VSPEC_OK) return r;
-        return launch_fold(p, p->nclusters, d_accum, nspectra, st);
+        return launch_fold(p, p->nclusters, d_accum, nspectra, st, 1, nullptr, true);
     }
     return VSPEC_OK;
 }
@@ -1785,10 +1816,14 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
     const int tilesB = p->N2 / p->RB;
     auto rows = [&](int sc) { return p->pair ? (sc + 1) / 2 : sc; };  // scratch spectra of sc spectra
     int slots = slots_for(p, (int)std::min<long long>(nB, (long long)tilesB * rows(sc_full)));
-    // a one-row transform in one launch: block k is the only writer of slot k
-    // and stores it, so nothing needs zeroing and the fold reads those slots
-    const bool store = p->fir_b && !p->kahan && !p->tc && nchunks == 1;
-    if (store) slots = (int)std::min<long long>(nB, (long long)tilesB * sc_full);
+    // A call of one launch: every slot a row launch uses has one writer, which
+    // stores it, and the fold reads only the slots that were written, so nothing
+    // needs zeroing (the memset cost 2 - 3 us of a 30 us call). One-row
+    // transforms: block k writes slot k, and the fold reads those.
+    const bool store = !p->kahan && !p->tc && nchunks == 1 && (p->fir_b || slots <= kFoldSlots);
+    const int gb_full = (int)std::min<long long>(nB, (long long)tilesB * rows(sc_full));
+    const vspec::SlotSpan written{gb_full, tilesB, rows(sc_full), 0, ilog2(p->RB)};
+    if (store && p->fir_b) slots = gb_full;
     if (!store) VSPEC_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)slots * p->N * accel, st));
     if (p->kahan) VSPEC_CUDA(cudaMemsetAsync(p->partial_comp, 0, (size_t)slots * p->N * accel, st));
 
@@ -1823,11 +1858,12 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
         const int gb = (int)std::min<long long>(nB, (long long)cb.tiles * rows(sc));
         // (a 2048-channel plan reports its one-pass kernel as such)
         const int kind = p->owner && p->owner->row_plan == p ? 3 : 1;
-        r = launch(p, kind, sc, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st);
+        r = launch(p, kind, sc, p->kernelB, dim3(gb), dim3(p->TB), argsB, p->smemB, st, 0, p->row_groups);
         if (r != VSPEC_OK) return r;
     }
     if (before_fold) VSPEC_CUDA(cudaStreamWaitEvent(st, before_fold, 0));
-    return launch_fold(p, slots, d_accum, nspectra, st);
+    return launch_fold(p, slots, d_accum, nspectra, st, 1, store && !p->fir_b ? &written : nullptr,
+                       !before_fold);
 }
 
 // The persistent ring form: one cooperative launch per kRingSlotsPerLaunch
@@ -2571,10 +2607,11 @@ extern "C" vspec_status vspec_execute_noalloc(const int8_t *d_in, int nchan, int
         VSPEC_CUDA(cudaLaunchKernel(c.kB, dim3(gb), dim3(c.TB), argsB, c.smemB, st));
     }
     const void *part = partial;
-    int groups = c.slots, stride = 1, N = c.N, N1 = c.N1, N2 = c.N2;  // at most 16 slots
+    vspec::SlotSpan span{0, 1, 1, c.slots, 0};
+    int stride = 1, N = c.N, N1 = c.N1, N2 = c.N2;  // at most 16 slots
     const int *ia = invA, *ib = invB;
     void *outp = d_accum;
-    void *argsR[] = {&part, &groups, &stride, &N, &N1, &N2, &ia, &ib, &outp};
+    void *argsR[] = {&part, &span, &stride, &N, &N1, &N2, &ia, &ib, &outp};
     VSPEC_CUDA(cudaLaunchKernel(c.kR, dim3((c.N + 31) / 32), dim3(32, 8), argsR, 0, st));
     return VSPEC_OK;
 }

@@ -38,6 +38,7 @@ struct ColBlk {
 };
 
 __global__ void __launch_bounds__(ColBlk::THREADS, 1) fir_colblk_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using G = ColBlk;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     P2 *data = reinterpret_cast<P2 *>(smem_raw);                         // [SPB][PTS]

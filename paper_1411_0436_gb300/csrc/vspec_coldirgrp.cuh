@@ -42,6 +42,7 @@ struct ColDirGrp {
 
 template <int N2_, int NPOL>
 __global__ void __launch_bounds__(512, 1) fir_coldirgrp_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using G = ColDirGrp<N2_>;
     constexpr int N2 = G::N2, PTS = G::PTS, C = G::C, TG = G::TG, R1 = G::R1, R2 = G::R2, M1 = G::M1, DEPTH = G::DEPTH;
     extern __shared__ __align__(16) unsigned char smem_raw[];

@@ -62,6 +62,7 @@ struct ColGrp {
 
 template <int N2_, int PT_, int GROUPS_, int NPOL>
 __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using G = ColGrp<N2_, PT_, GROUPS_>;
     constexpr int N2 = G::N2, PT = G::PT, PTS = G::PTS, C = G::C, TG = G::TG, KP = G::KP, SPB = G::SPB, RING = G::RING,
                   SS = G::SS, R1 = G::R1, R2 = G::R2, M1 = G::M1;
@@ -111,34 +112,6 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
         const int w0 = x * C;  // first column (or word) of the tile
         auto column = [&](int c) { return (w0 + c) >> p.lsub; };
         auto zcol = [&](int c) { return (p.lsub ? (size_t)((w0 + c) & (p.nsub - 1)) * p.N : 0) + column(c); };
-
-        // the run's coefficients and four-step twiddles, into this thread's lane
-        {
-            uint32_t v[32];
-#pragma unroll
-            for (int i = 0; i < 32; i++) v[i] = 0u;
-#pragma unroll
-            for (int k = 0; k < KP; k++) {
-                const int pt = t + TG * k;
-                const float *h = p.coef + column(pt % C) + (size_t)p.N1 * (pt / C);
-#pragma unroll
-                for (int i = 0; i < PT; i++)
-                    if (i >= D) v[k * PT + i] = __float_as_uint(__ldg(h + (size_t)(i - D) * p.N));
-            }
-            tmem_st32(tm, v);
-#pragma unroll
-            for (int i = 0; i < G::NC; i++) {
-                const int e = t + TG * i, c = e % C, row0 = G::kOnePass ? 0 : (e / C) % R1 * R2;
-#pragma unroll
-                for (int q = 0; q < G::NT; q++) {
-                    const float2 w = __ldg(p.twZ + (size_t)(row0 + q) * p.N1 + column(c));
-                    v[2 * (i * G::NT + q)] = __float_as_uint(w.x);
-                    v[2 * (i * G::NT + q) + 1] = __float_as_uint(w.y);
-                }
-            }
-            tmem_st32(tm + 32, v);
-            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
-        }
 
         // Ring slot (fr - first) mod RING holds absolute frame fr, first the
         // oldest frame of the run's first spectrum (frames before the input are
@@ -192,7 +165,36 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
+        // (the last run's readers of the ring are past its last barrier)
         stage(0, PT - 1 + min(SPB, s_end - s_beg), 0);
+
+        // the run's coefficients and four-step twiddles, into this thread's lane
+        {
+            uint32_t v[32];
+#pragma unroll
+            for (int i = 0; i < 32; i++) v[i] = 0u;
+#pragma unroll
+            for (int k = 0; k < KP; k++) {
+                const int pt = t + TG * k;
+                const float *h = p.coef + column(pt % C) + (size_t)p.N1 * (pt / C);
+#pragma unroll
+                for (int i = 0; i < PT; i++)
+                    if (i >= D) v[k * PT + i] = __float_as_uint(__ldg(h + (size_t)(i - D) * p.N));
+            }
+            tmem_st32(tm, v);
+#pragma unroll
+            for (int i = 0; i < G::NC; i++) {
+                const int e = t + TG * i, c = e % C, row0 = G::kOnePass ? 0 : (e / C) % R1 * R2;
+#pragma unroll
+                for (int q = 0; q < G::NT; q++) {
+                    const float2 w = __ldg(p.twZ + (size_t)(row0 + q) * p.N1 + column(c));
+                    v[2 * (i * G::NT + q)] = __float_as_uint(w.x);
+                    v[2 * (i * G::NT + q) + 1] = __float_as_uint(w.y);
+                }
+            }
+            tmem_st32(tm + 32, v);
+            asm volatile("tcgen05.wait::st.sync.aligned;" ::: "memory");
+        }
         int r0 = 0;  // ring slot of the batch's oldest frame
         for (int s = s_beg; s < s_end; s += SPB) {
             const int nb = min(SPB, s_end - s);

@@ -370,6 +370,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_kernel(const __grid_constan
         }
         row_fft_detect<LOGN1>(rowbuf, p, acc);  // last spectrum
     }
+    pdl_trigger();
     // no CTA may leave while others can still read its tiles
     cluster.sync();
 

@@ -354,6 +354,7 @@ __global__ void __launch_bounds__(kThreads, 1) fused_w_kernel(const __grid_const
         __syncthreads();
         rows_detect(rowbuf, twr, tw2, warp, lane, acc);  // last spectrum
     }
+    pdl_trigger();
     cluster.sync();
 
     if constexpr (PT > 1) {

@@ -121,6 +121,27 @@ struct RowParams {
     long long nframes;   // frames the call's input holds (bounds checks of debug builds)
 };
 
+// ------------------------------------------------------ dependent launches --
+// The kernels of a call follow one another as programmatic dependent launches:
+// a kernel's CTAs may be placed once every CTA of the one before has started
+// (pdl_trigger), each as an SM frees up, and run their prologue there; pdl_wait
+// returns when all of that kernel is done and its writes are visible. A kernel
+// launched that way waits before it reads what the kernel before wrote, in
+// every CTA, so that its own end implies that kernel's. Both are no-ops in an
+// ordinary launch.
+//
+// Kernel A triggers at its start: kernel B's CTAs take a whole SM each, so they
+// only start where one is free. (Smaller CTAs would pile up on the SMs that
+// finish first: row4096_kernel 382 -> 500 us, so it is launched in the ordinary
+// way.) The kernels before a fold trigger at their end: fold CTAs placed earlier
+// gather on the idle SMs and read all slots from there (a 2-point-column call
+// of 257 spectra 33 -> 48 us). Whole calls, GB300, us, ordinary launches with a
+// memset of the slots against this: PFB 65536 channels 5 spectra 34.8 / 24.6, 40
+// spectra 57.3 / 46.7, 257 spectra 175 / 160; 4096 channels, 5 spectra on the
+// cluster kernel 21.5 / 17.4; 32768 channels, 1000 spectra 273 / 262.
+__device__ __forceinline__ void pdl_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+
 // ------------------------------------------------------------ work split --
 // A launch's work is tiles x sc (tile, spectrum) items, tile-major. Block k
 // of n takes items [k T / n, (k+1) T / n), T = tiles * sc: equal shares to
@@ -141,6 +162,20 @@ __device__ __forceinline__ int span_slot(int tiles, int sc, int x) {
     const long long T = (long long)tiles * sc;
     const long long k_lo = (((long long)x * sc + 1) * gridDim.x - 1) / T;
     return (int)(blockIdx.x - k_lo);
+}
+
+// Slots of row tile x that a launch of n blocks (at most one per item) wrote:
+// the blocks between those that hold the tile's first and last item, ranks 0 ..
+// .. n = 0: `all` slots (zeroed, or every one written).
+struct SlotSpan {
+    int n, tiles, sc, all;
+    int lrb;  // log2 rows per tile
+};
+__device__ __forceinline__ int span_slots(const SlotSpan &w, int row) {
+    if (w.n == 0) return w.all;
+    const unsigned long long T = (unsigned long long)w.tiles * w.sc, x = row >> w.lrb;
+    const unsigned long long k_lo = ((x * w.sc + 1) * w.n - 1) / T, k_hi = ((x + 1) * w.sc * w.n - 1) / T;
+    return (int)(k_hi - k_lo) + 1;
 }
 
 // Kernel A's split: blocks come in groups of G consecutive blocks that take
@@ -449,6 +484,7 @@ __device__ __forceinline__ void fir_colfft_segment(const ColParams &p, typename 
 
 template <int NPOL, int PT, int PPT>
 __global__ void __launch_bounds__(512) fir_colfft_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using T = typename Elem<NPOL>::T;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     T *data = reinterpret_cast<T *>(smem_raw);  // [PT][N2][C]
@@ -683,6 +719,7 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
 
 template <int N2, int R1 = N2>
 __global__ void __launch_bounds__(512, 1) fir_colreg_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
     const TileSplit sp = tile_split(p.tiles, p.sc, p.G);
     bool first = true;
@@ -892,6 +929,7 @@ __global__ void __launch_bounds__(512) fir_coldir_kernel(const __grid_constant__
 // the block walks its consecutive spectra), the coefficients from L1/L2.
 template <int NPOL, int PPT>
 __global__ void __launch_bounds__(512) fir_colfft_gather_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using T = typename Elem<NPOL>::T;
     constexpr int NC = 2 * NPOL;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1116,6 +1154,7 @@ __host__ __device__ constexpr size_t row_ring_bytes(int npol, int P, int N1) {
 
 template <int NPOL, bool KAHAN = false, bool FIR = false>
 __global__ void __launch_bounds__(256, 2) rowfft_detect_kernel(const __grid_constant__ RowParams p) {
+    pdl_wait();
     using T = typename Elem<NPOL>::T;
     using A = typename Elem<NPOL>::Acc;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1242,6 +1281,7 @@ __global__ void __launch_bounds__(256, 2) rowfft_detect_kernel(const __grid_cons
         flush(first);
         __syncthreads();  // acc is zeroed again by the next segment
     }
+    pdl_trigger();
 }
 
 // ------------------------------------------------------ kernel B, 2048 --
@@ -1390,6 +1430,7 @@ __device__ __forceinline__ void row2048_last(const typename Elem<NPOL>::T *row, 
 
 template <int NPOL, bool KAHAN, bool FIR, bool ZSPLIT = false>
 __global__ void __launch_bounds__(256, KAHAN ? 1 : 2) row2048_kernel(const __grid_constant__ RowParams p) {
+    pdl_wait();
     using T = typename Elem<NPOL>::T;
     using A = typename Elem<NPOL>::Acc;
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -1460,6 +1501,7 @@ __global__ void __launch_bounds__(256, KAHAN ? 1 : 2) row2048_kernel(const __gri
         }
         flush(first);
     }
+    pdl_trigger();
 }
 
 // Kernel B for 4096-point rows (dual-pol, no pre-filter; 2^19 PFB plans):
@@ -1474,6 +1516,7 @@ constexpr int kRow4096Stride = 4096 + 4096 / 8;
 
 template <bool ZSPLIT = false>
 __global__ void __launch_bounds__(512, 1) row4096_kernel(const __grid_constant__ RowParams p) {
+    pdl_wait();
     using A = float4;
     extern __shared__ __align__(16) unsigned char smem_raw[];
     P2 *row = reinterpret_cast<P2 *>(smem_raw);  // one row, pad8 layout
@@ -1561,6 +1604,7 @@ __global__ void __launch_bounds__(512, 1) row4096_kernel(const __grid_constant__
         }
         flush(first);
     }
+    pdl_trigger();
 }
 
 // ------------------------------------------------------------ sub-bands --
@@ -1596,6 +1640,8 @@ __global__ void deinterleave_kernel(const W *in, W *out, int nsub, long long M, 
 // 32 positions x 8 slot lanes; gridDim (ceil(N / 32), groups of 16).
 template <int NPOL, bool KAHAN>
 __global__ void __launch_bounds__(256) fold_slots_kernel(void *partial, void *partial_comp, int slots, int N) {
+    pdl_trigger();
+    pdl_wait();
     using A = typename Elem<NPOL>::Acc;
     __shared__ A lane_sum[8][32];
     __shared__ A lane_comp[8][32];
@@ -1674,7 +1720,7 @@ __global__ void __launch_bounds__(256) fold_slots_kernel(void *partial, void *pa
 // most 512: PB = 32 runs two elements per thread); the short form, with more
 // CTAs and lanes, is for small N2 with many slots.
 template <int NPOL, int PB, int L>
-__global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, int groups, int stride, int N,
+__global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, const SlotSpan span, int stride, int N,
                                                          int N2, const int *invA, void *out) {
     using A = typename Elem<NPOL>::Acc;
     constexpr int Q2G = PB / 8;  // q2 values per block
@@ -1684,15 +1730,38 @@ __global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, in
     const int k2_0 = 16 * (blockIdx.x % nk);
     const int q1 = (blockIdx.x / nk) % 16, g = blockIdx.x / (nk * 16);
     const int p0 = 128 * q1 + PB * g;
+    constexpr int TH = E * L < 512 ? E * L : PB == 32 ? 256 : 512;  // threads (launch_fold)
     const A *pp = reinterpret_cast<const A *>(partial) + (size_t)blockIdx.y * N;  // band blockIdx.y of every slot
-    for (int e = threadIdx.x; e < E * L; e += blockDim.x) {
-        const int l = e / E, r = (e % E) / PB, j = e % PB;
-        const size_t idx = (size_t)__ldg(invA + k2_0 + r) * 2048 + p0 + j;
+    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N;
+    // what does not depend on the kernel before: slot counts, the accumulators
+    constexpr int NI = E * L / TH, NO = (E + TH - 1) / TH;
+    size_t idx[NI];
+    int groups[NI];
+#pragma unroll
+    for (int i = 0; i < NI; i++) {
+        const int e = threadIdx.x + TH * i, r = (e % E) / PB, j = e % PB;
+        const int row = __ldg(invA + k2_0 + r);
+        groups[i] = span_slots(span, blockIdx.y * N2 + row);
+        idx[i] = (size_t)row * 2048 + p0 + j;
+    }
+    size_t k[NO];
+    A a[NO];
+#pragma unroll
+    for (int i = 0; i < NO; i++) {
+        const int e = threadIdx.x + TH * i, r = e & 15, j = e >> 4;  // position offset j = 8 (q2 - Q2G g) + q3
+        const int k1 = q1 + 16 * (Q2G * g + (j >> 3)) + 256 * (j & 7);
+        k[i] = (size_t)k1 * N2 + k2_0 + r;
+        if (e < E) a[i] = o[k[i]];
+    }
+    pdl_wait();
+#pragma unroll
+    for (int i = 0; i < NI; i++) {
+        const int e = threadIdx.x + TH * i, l = e / E, r = (e % E) / PB, j = e % PB;
         A s;
         if constexpr (NPOL == 2) s = make_float4(0.f, 0.f, 0.f, 0.f);
         else s = 0.f;
-        for (int gs = l; gs < groups; gs += L) {
-            const A v = pp[(size_t)gs * stride * N + idx];
+        for (int gs = l; gs < groups[i]; gs += L) {
+            const A v = pp[(size_t)gs * stride * N + idx[i]];
             if constexpr (NPOL == 2) {
                 s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
             } else {
@@ -1702,11 +1771,10 @@ __global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, in
         tile[l][r][j] = s;
     }
     __syncthreads();
-    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N;
-    for (int e = threadIdx.x; e < E; e += blockDim.x) {
-        const int r = e & 15, j = e >> 4;  // position offset j = 8 (q2 - Q2G g) + q3
-        const int k1 = q1 + 16 * (Q2G * g + (j >> 3)) + 256 * (j & 7);
-        const size_t k = (size_t)k1 * N2 + k2_0 + r;
+#pragma unroll
+    for (int i = 0; i < NO; i++) {
+        const int e = threadIdx.x + TH * i, r = e & 15, j = e >> 4;
+        if (e >= E) break;
         A v = tile[0][r][j];
 #pragma unroll
         for (int l = 1; l < L; l++) {
@@ -1717,13 +1785,59 @@ __global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, in
                 v += w;
             }
         }
+        if constexpr (NPOL == 2) o[k[i]] = make_float4(a[i].x + v.x, a[i].y + v.y, a[i].z + v.z, a[i].w + v.w);
+        else o[k[i]] = a[i] + v;
+    }
+}
+
+// The same for N2 < 16, where rows are split over many CTAs (up to 78 slots):
+// a block takes 4 consecutive channels of 8 values of q3 (m = q1 N2 + k2 = 4 b
+// .. + 3 of one q2), 8 contiguous positions of each row it meets, with 16 slot
+// lanes per element, added in lane order. 64 N2 blocks of 512 threads. (The
+// channel-order fold below reads scattered 16-byte pieces with 8 lanes.)
+template <int NPOL>
+__global__ void __launch_bounds__(512) reduce2048_short_kernel(const void *partial, const SlotSpan span, int stride,
+                                                               int N, int N2, const int *invA, void *out) {
+    using A = typename Elem<NPOL>::Acc;
+    __shared__ A tile[16][32];
+    const int l = threadIdx.x >> 5, e = threadIdx.x & 31;  // lane; element, q3 fastest
+    const int m = 4 * (blockIdx.x % (4 * N2)) + (e >> 3), q2 = blockIdx.x / (4 * N2), q3 = e & 7;
+    const int row = __ldg(invA + m % N2), groups = span_slots(span, blockIdx.y * N2 + row);
+    const A *pp = reinterpret_cast<const A *>(partial) + (size_t)blockIdx.y * N + (size_t)row * 2048 + 128 * (m / N2) +
+                  8 * q2 + q3;
+    // (written out by element e' = 4 q3 + channel, for runs of consecutive channels)
+    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N + 4 * (blockIdx.x % (4 * N2)) + (e & 3) +
+           (size_t)16 * N2 * q2 + (size_t)256 * N2 * (e >> 2);
+    A s;
+    if constexpr (NPOL == 2) s = make_float4(0.f, 0.f, 0.f, 0.f);
+    else s = 0.f;
+    A a = s;
+    if (l == 0) a = *o;
+    pdl_wait();
+    for (int g = l; g < groups; g += 16) {
+        const A v = pp[(size_t)g * stride * N];
         if constexpr (NPOL == 2) {
-            const float4 a = o[k];
-            o[k] = make_float4(a.x + v.x, a.y + v.y, a.z + v.z, a.w + v.w);
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
         } else {
-            o[k] += v;
+            s += v;
         }
     }
+    tile[l][e] = s;
+    __syncthreads();
+    if (l) return;
+    const int src = 8 * (e & 3) + (e >> 2);
+    s = tile[0][src];
+#pragma unroll
+    for (int i = 1; i < 16; i++) {
+        const A v = tile[i][src];
+        if constexpr (NPOL == 2) {
+            s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
+        } else {
+            s += v;
+        }
+    }
+    if constexpr (NPOL == 2) *o = make_float4(a.x + s.x, a.y + s.y, a.z + s.z, a.w + s.w);
+    else *o = a + s;
 }
 
 // Fold of the partial-sum slots into the caller's accumulator, with the
@@ -1732,7 +1846,7 @@ __global__ void __launch_bounds__(512) reduce2048_kernel(const void *partial, in
 // A block is 32 channels x 8 slot lanes (blockDim (32, 8)): lane y sums
 // slots y, y + 8, ..., and lane 0 adds the eight lane sums in order.
 template <int NPOL>
-__global__ void __launch_bounds__(256) reduce_kernel(const void *partial, int groups, int stride, int N, int N1,
+__global__ void __launch_bounds__(256) reduce_kernel(const void *partial, const SlotSpan span, int stride, int N, int N1,
                                                      int N2, const int *invA, const int *invB, void *out) {
     using A = typename Elem<NPOL>::Acc;
     __shared__ A lane_sum[8][32];
@@ -1742,10 +1856,20 @@ __global__ void __launch_bounds__(256) reduce_kernel(const void *partial, int gr
     A s;
     if constexpr (NPOL == 2) s = make_float4(0.f, 0.f, 0.f, 0.f);
     else s = 0.f;
+    // what does not depend on the kernel before: slot count, position, the accumulator
     size_t idx = 0;
+    int groups = 0;
+    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N;
+    A a = s;
     if (k < N) {
         const int k2 = k & (N2 - 1), k1 = k / N2;
-        idx = (size_t)__ldg(invA + k2) * N1 + __ldg(invB + k1);
+        const int row = __ldg(invA + k2);
+        groups = span_slots(span, blockIdx.y * N2 + row);
+        idx = (size_t)row * N1 + __ldg(invB + k1);
+        if (y == 0) a = o[k];
+    }
+    pdl_wait();
+    if (k < N) {
         for (int g = y; g < groups; g += 8) {
             const A v = pp[(size_t)g * stride * N + idx];
             if constexpr (NPOL == 2) {
@@ -1758,7 +1882,6 @@ __global__ void __launch_bounds__(256) reduce_kernel(const void *partial, int gr
     lane_sum[y][threadIdx.x] = s;
     __syncthreads();
     if (y != 0 || k >= N) return;
-    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N;
 #pragma unroll
     for (int l = 1; l < 8; l++) {
         const A v = lane_sum[l][threadIdx.x];
@@ -1768,12 +1891,8 @@ __global__ void __launch_bounds__(256) reduce_kernel(const void *partial, int gr
             s += v;
         }
     }
-    if constexpr (NPOL == 2) {
-        const float4 a = o[k];
-        o[k] = make_float4(a.x + s.x, a.y + s.y, a.z + s.z, a.w + s.w);
-    } else {
-        o[k] += s;
-    }
+    if constexpr (NPOL == 2) o[k] = make_float4(a.x + s.x, a.y + s.y, a.z + s.z, a.w + s.w);
+    else o[k] = a + s;
 }
 
 // Compensated fold: each lane keeps a Kahan sum of its slots' compensated
@@ -1785,6 +1904,7 @@ __global__ void __launch_bounds__(256) reduce_kahan_kernel(const void *partial, 
                                                            int groups, int stride, int N, int N1, int N2,
                                                            const int *invA, const int *invB, void *out,
                                                            void *out_comp) {
+    pdl_wait();
     using A = typename Elem<NPOL>::Acc;
     __shared__ A lane_sum[8][32];
     const int k = blockIdx.x * 32 + threadIdx.x;

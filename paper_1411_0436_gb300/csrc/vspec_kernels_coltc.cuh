@@ -178,6 +178,7 @@ __host__ __device__ constexpr uint32_t instr_desc_f16(int m, int n) {
 
 template <int N2>
 __global__ void __launch_bounds__(512, 1) fir_coltc_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using G = ColTc<N2>;
     using namespace tc;
     constexpr int PT = G::PT, PTS = G::PTS, C = G::C, SPB = G::SPB;

@@ -127,6 +127,7 @@ __device__ __forceinline__ void unpack_half2(uint32_t w, uint32_t &x, uint32_t &
 
 template <int Q>
 __global__ void __launch_bounds__(512, 1) fir_tcfir_kernel(const __grid_constant__ ColParams p) {
+    pdl_trigger();
     using G = TcFir<Q>;
     using namespace tc;
     constexpr int M = G::M, ROWS = G::ROWS, RS = G::RS, N2 = G::N2;

@@ -99,14 +99,15 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
                      :: "r"(tc::smem_addr(tmem_slot)), "r"(G::TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
+    for (int e = tid; e < G::TW2; e += G::THREADS) tw2s[e] = __ldg(p.twBt + G::TW1 + e);
     if (tid == 0) {
         *gave_up = 0;
         for (int b = 0; b < G::NBUF; b++) tc::mbar_init(full + b, 1);
         asm volatile("fence.mbarrier_init.release.cluster;" ::: "memory");
+        pdl_wait();  // kernel A's rows
         tc::fence_proxy_async();
         for (int i = 0; i < min(n, G::NBUF); i++) issue(i);
     }
-    for (int e = tid; e < G::TW2; e += G::THREADS) tw2s[e] = __ldg(p.twBt + G::TW1 + e);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory");
@@ -304,6 +305,7 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
             }
         }
     }
+    pdl_trigger();
     if (*gave_up && tid == 0)  // no copy may land after the CTA has left
         for (int b = 0; b < min(n, G::NBUF); b++) tc::mbar_wait(full + b, (copied[b] / G::NBUF) & 1);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");

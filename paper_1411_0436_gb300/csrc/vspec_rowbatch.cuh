@@ -299,6 +299,7 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             // (the next batch's first barrier orders these reads before data is written)
         }
     }
+    pdl_trigger();
     if constexpr (NPOL == 2) {
         asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
         __syncthreads();
@@ -329,6 +330,11 @@ __global__ void __launch_bounds__(512) fold_row_kernel(const void *partial, int 
     A s;
     if constexpr (NPOL == 2) s = make_float4(0.f, 0.f, 0.f, 0.f);
     else s = 0.f;
+    const int q3 = pos & 7, q2 = (pos >> 3) % R2, q1 = pos / (8 * R2);
+    A *o = reinterpret_cast<A *>(out) + q1 + R1 * (q2 + R2 * q3);
+    A a = s;
+    if (ty == 0) a = *o;
+    pdl_wait();
     for (int g = ty; g < slots; g += 64) add(s, pp[(size_t)g * N]);
     lane_sum[ty][tx] = s;
     __syncthreads();
@@ -343,9 +349,6 @@ __global__ void __launch_bounds__(512) fold_row_kernel(const void *partial, int 
     if (ty) return;
 #pragma unroll
     for (int l = 1; l < 8; l++) add(s, lane_sum[l][tx]);
-    const int q3 = pos & 7, q2 = (pos >> 3) % R2, q1 = pos / (8 * R2);
-    A *o = reinterpret_cast<A *>(out) + q1 + R1 * (q2 + R2 * q3);
-    A a = *o;
     add(a, s);
     *o = a;
 }
