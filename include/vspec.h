@@ -329,8 +329,8 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  *                            16 taps), register columns (dual-pol direct), the
  *                            general kernel (general-paired: two single-pol
  *                            spectra at once), taps read from the
- *                            input (gather-blocked: from frames staged in
- *                            shared memory); none for one-row transforms
+ *                            input (gather-blocked: columns of the longest
+ *                            transforms, from frames staged in shared memory); none for one-row transforms
  *   B=row2048|general|tensor kernel B's form (-batched: the one-row kernel of
  *                            512, 1024 and 2048 channels)
  *   fir-in-B                 one-row transform: the FIR runs in kernel B

@@ -27,7 +27,6 @@
 #include "vspec_kernels_tcfir.cuh"
 #include "vspec_ring.cuh"
 #include "vspec_row2048.cuh"
-#include "vspec_colblk.cuh"
 #include "vspec_bp.cuh"
 #include "vspec_internal.h"
 
@@ -46,6 +45,9 @@ cudaError_t vspec_colgrp16_debug_flags(unsigned *flags, bool clear);
 // vspec_coldirgrp.cu
 const void *vspec_pick_kernel_coldirgrp(int N2, int npol, size_t *smem, int *groups);
 cudaError_t vspec_coldirgrp_debug_flags(unsigned *flags, bool clear);
+// vspec_colblk.cu
+const void *vspec_pick_kernel_colblk(int N2, int npol, int P, size_t *smem);
+cudaError_t vspec_colblk_debug_flags(unsigned *flags, bool clear);
 // vspec_rowbatch.cu
 const void *vspec_pick_kernel_rowbatch(int nchan, int npol, int P, size_t *smem);
 const void *vspec_pick_fold_row(int npol);
@@ -792,6 +794,19 @@ vspec_status build_plan(vspec_plan *p) {
             PT = p->P <= 4 ? 4 : p->P <= 8 ? 8 : 16;
         }
     }
+    // the longest transforms, with 2048-point rows: the blocked kernel A (2^20
+    // channels; single-pol pre-filters from 2^18 on, whose grouped kernel would
+    // have 8-byte tile rows)
+    size_t smem_colblk = 0;
+    const void *colblk = nullptr;
+    if (!p->req_n2 && !p->req_cols && (N == 1 << 20 || (p->npol == 1 && pfb && N >= 1 << 18)) &&
+        (p->npol == 2 || !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR)))) {
+        colblk = vspec_pick_kernel_colblk(N / kRowElems, p->npol, p->P, &smem_colblk);
+        if (colblk) {
+            N2 = N / kRowElems;
+            p->gather = false;
+        }
+    }
     const int N1 = N / N2;
     if (N1 > 4096) {
         g_last_error = "nchan too large for this mode in this build";
@@ -816,12 +831,7 @@ vspec_status build_plan(vspec_plan *p) {
     const bool colreg_tiles = colgrp || (p->npol == 2 && pfb && PT == 8 && !p->gather && (N1 == 2048 || N1 == 4096) &&
                                          N2 >= 2 && N2 <= 128 && !p->req_cols);
     if (colreg_tiles) C = 512 / N2;
-    // dual-pol PFB too long for a register window, 512-point columns (2^20):
-    // the blocked kernel A, up to its 8 taps (0.78 against 1.77 ms per 100
-    // spectra; the gather kernel keeps 9 .. 16 taps and single polarisation)
-    const bool colblk = p->npol == 2 && p->gather && p->P <= vspec::ColBlk::PT && N2 == vspec::ColBlk::N2 &&
-                        N1 >= vspec::ColBlk::C && !p->req_cols;
-    if (colblk) C = vspec::ColBlk::C;
+    if (colblk) C = 2048 / N2;
     if (p->req_cols) {  // a requested tile width: the general kernel A
         const int c = p->req_cols;
         if (!is_pow2(c) || c < cmin || c > N1 || (long long)c * N2 > 4096 || N2 == 1) {
@@ -845,14 +855,14 @@ vspec_status build_plan(vspec_plan *p) {
     p->kernelA = p->gather ? (p->npol == 2 ? pick_kernel_gather<2>(PPT) : pick_kernel_gather<1>(PPT))
                            : (p->npol == 2 ? pick_kernel_a<2>(PT, PPT) : pick_kernel_a<1>(PT, PPT));
     // single polarisation in these forms: two spectra per scratch element
-    p->pair = p->npol == 1 && (coldir || colgrp);
+    p->pair = p->npol == 1 && (coldir || colgrp || colblk);
     if (coldir) {
         p->kernelA = coldir;
         p->formA = p->pair ? "general-paired" : "coldir";
     }
     if (p->gather) p->formA = "gather";
     if (colblk) {
-        p->kernelA = (const void *)vspec::fir_colblk_kernel;
+        p->kernelA = colblk;
         p->formA = "gather-blocked";
     }
     if (!p->kernelA) {
@@ -920,7 +930,7 @@ vspec_status build_plan(vspec_plan *p) {
     // sums or tensor-core rows: four radix-8 passes (row4096_kernel)
     const bool row4096 = N1 == 4096 && p->npol == 2 && !p->fir_b &&
                          !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8));
-    const std::vector<int> rA = colblk ? std::vector<int>{8, 8, 8} : (tcfir || coltc) ? std::vector<int>{N2} : colreg ? r_colreg : coldir ? r_coldir
+    const std::vector<int> rA = colblk ? std::vector<int>{8, N2 / 64, 8} : (tcfir || coltc) ? std::vector<int>{N2} : colreg ? r_colreg : coldir ? r_coldir
                                                                                : radix_list(e2, maxbitsA),
                            rB = row4096 ? std::vector<int>{8, 8, 8, 8} : radix_list(e1);
     int twA_n = 0, twB_n = 0;
@@ -963,7 +973,7 @@ vspec_status build_plan(vspec_plan *p) {
     p->smemA = (size_t)PT * N2 * C * elem + (size_t)N2 * C * sizeof(float2) +
                (!p->gather ? 2 * (size_t)PT * N2 * C * p->npol * 2 : 0);
     if (colreg) p->smemA = smem_colreg;
-    if (colblk) p->smemA = vspec::ColBlk::smem;
+    if (colblk) p->smemA = smem_colblk;
     if (tcfir || coltc) p->smemA = smem_tcA;
     if (coldir) p->smemA = smem_coldir;
     p->smemB = (size_t)p->RB * (N1 + (N1 >> 4)) * elem + (size_t)p->RB * N1 * accel;
@@ -2239,7 +2249,7 @@ vspec_status vspec_debug_flags(unsigned *flags, int clear) {
     VSPEC_CUDA(vspec_rowbatch_debug_flags(&row_flags, clear != 0));
     *flags |= ring_flags | bp_flags | row_flags;
     for (auto fn : {vspec_colgrp4_debug_flags, vspec_colgrp8_debug_flags, vspec_colgrp16_debug_flags,
-                    vspec_coldirgrp_debug_flags}) {
+                    vspec_coldirgrp_debug_flags, vspec_colblk_debug_flags}) {
         unsigned f = 0;
         VSPEC_CUDA(fn(&f, clear != 0));
         *flags |= f;
