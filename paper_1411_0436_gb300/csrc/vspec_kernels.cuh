@@ -119,6 +119,7 @@ struct RowParams {
     long long s0;        // absolute index of the chunk's first spectrum
     int store;           // 1: every slot has exactly one writer this call, which stores (no zeroing)
     long long nframes;   // frames the call's input holds (bounds checks of debug builds)
+    long long band_bytes;  // row_batch_kernel: input of band b (of `tiles`) at b * band_bytes
 };
 
 // ------------------------------------------------------ dependent launches --

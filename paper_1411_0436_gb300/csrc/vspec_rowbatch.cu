@@ -6,13 +6,8 @@
 
 namespace {
 template <int N, int NPOL, int PT> const void *instance(size_t *smem) {
-    using G = vspec::RowBatch<N, NPOL, PT>;
-    if constexpr (G::smem <= 232448) {
-        *smem = G::smem;
-        return (const void *)vspec::row_batch_kernel<N, NPOL, PT>;
-    } else {
-        return nullptr;  // 2048 channels, dual-pol, more than 8 taps: the ring does not fit
-    }
+    *smem = vspec::RowBatch<N, NPOL, PT>::smem;
+    return (const void *)vspec::row_batch_kernel<N, NPOL, PT>;
 }
 template <int N, int NPOL> const void *by_taps(int P, size_t *smem) {
     return P <= 1 ? instance<N, NPOL, 1>(smem) : P <= 8 ? instance<N, NPOL, 8>(smem) : instance<N, NPOL, 16>(smem);

@@ -29,7 +29,7 @@
 // Measured (GB300, whole calls, us): 1024 channels dual-pol 8 taps 2048 spectra
 // 66 -> 22.6, 4096 spectra 114 -> 35, direct 60 -> 29; single-pol 4096 spectra
 // 72 -> 21; 2048 channels 4096 spectra 103 -> 64 (against the cluster kernel),
-// direct 91 -> 47; the others against the general row kernel, which unpacked
+// direct 91 -> 47; dual-pol 16 taps 257 spectra 37 -> 20.5, 4096 179 -> 98; the others against the general row kernel, which unpacked
 // every tap of every spectrum and kept its sums in shared memory.
 #pragma once
 #include "vspec_kernels.cuh"
@@ -39,7 +39,9 @@ namespace vspec {
 
 template <int N_, int NPOL_, int PT_>
 struct RowBatch {
-    static constexpr int N = N_, NPOL = NPOL_, PT = PT_, THREADS = 512, SPB = 8192 / N;
+    // (2048 channels, dual-pol, more than 8 taps: two spectra, the ring takes the room)
+    static constexpr int N = N_, NPOL = NPOL_, PT = PT_, THREADS = 512,
+                         SPB = N == 2048 && NPOL == 2 && PT > 8 ? 2 : 8192 / N;
     static constexpr int R1 = N == 512 ? 8 : 16, R2 = N == 2048 ? 16 : 8;  // then radix 8
     static constexpr int M1 = N / R1, KP = N / THREADS;   // first-pass stride; points per thread
     static constexpr int BS = NPOL == 2 ? SPB : 2 * SPB;  // spectra per batch
@@ -74,8 +76,10 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
         }
     }
-    const Span sp = block_span(1, p.sc);
-    const int s_beg = (int)sp.lo, s_end = (int)sp.hi;
+    // p.tiles bands (see run_rows): an equal share of one band's spectra
+    const int per = gridDim.x / p.tiles, rank = blockIdx.x % per;
+    const int8_t *in = p.in + (long long)(blockIdx.x / per) * p.band_bytes;
+    const int s_beg = (int)((long long)p.sc * rank / per), s_end = (int)((long long)p.sc * (rank + 1) / per);
     // Ring slot (fr - first) mod RING holds absolute frame fr, first the oldest
     // frame of the run's first spectrum (D leading taps have zero coefficients;
     // frames before the input are clamped).
@@ -88,7 +92,7 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
             if (fr < 0) fr = 0;
             int sl = slot + u;
             if (sl >= RING) sl -= RING;
-            const unsigned char *src = reinterpret_cast<const unsigned char *>(p.in) + (fr * N) * W + 16 * e;
+            const unsigned char *src = reinterpret_cast<const unsigned char *>(in) + (fr * N) * W + 16 * e;
             if (dbg_ok(fr < p.nframes, kDbgInput))
                 asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
                              :: "r"(tc::smem_addr(ring + (size_t)sl * N * W + 16 * e)), "l"(src) : "memory");
@@ -311,7 +315,8 @@ __global__ void __launch_bounds__(512, 1) row_batch_kernel(const __grid_constant
 // Fold of the one-row transforms' slots: position pos = M1 q1 + 8 q2 + q3 of
 // every slot is channel q1 + R1 (q2 + R2 q3). A block is 8 positions x 64 slot
 // lanes: lane y sums slots y, y + 64, ..., then eight threads of each position
-// add eight lane sums in order, then one adds those eight. (The general fold
+// add eight lane sums in order, then one adds those eight. Band blockIdx.y has
+// the slots blockIdx.y * slots .. (The general fold
 // takes two launches over as many slots and 32-channel blocks that leave most
 // SMs idle at these sizes.)
 template <int NPOL>
@@ -319,7 +324,7 @@ __global__ void __launch_bounds__(512) fold_row_kernel(const void *partial, int 
     using A = typename Elem<NPOL>::Acc;
     __shared__ A lane_sum[64][8];
     const int tx = threadIdx.x, ty = threadIdx.y, pos = blockIdx.x * 8 + tx;
-    const A *pp = reinterpret_cast<const A *>(partial) + pos;
+    const A *pp = reinterpret_cast<const A *>(partial) + (size_t)blockIdx.y * slots * N + pos;
     auto add = [](A &s, const A &v) {
         if constexpr (NPOL == 2) {
             s.x += v.x; s.y += v.y; s.z += v.z; s.w += v.w;
@@ -331,7 +336,7 @@ __global__ void __launch_bounds__(512) fold_row_kernel(const void *partial, int 
     if constexpr (NPOL == 2) s = make_float4(0.f, 0.f, 0.f, 0.f);
     else s = 0.f;
     const int q3 = pos & 7, q2 = (pos >> 3) % R2, q1 = pos / (8 * R2);
-    A *o = reinterpret_cast<A *>(out) + q1 + R1 * (q2 + R2 * q3);
+    A *o = reinterpret_cast<A *>(out) + (size_t)blockIdx.y * N + q1 + R1 * (q2 + R2 * q3);
     A a = s;
     if (ty == 0) a = *o;
     pdl_wait();
