@@ -39,6 +39,8 @@ cudaError_t vspec_ring_debug_flags(unsigned *flags, bool clear);
 const void *vspec_pick_kernel_colgrp4(int N2, int npol, size_t *smem, int *groups);
 const void *vspec_pick_kernel_colgrp8(int N2, int npol, size_t *smem, int *groups);
 const void *vspec_pick_kernel_colgrp16(int N2, int npol, size_t *smem, int *groups);
+const void *vspec_pick_kernel_colgrp4_bands(int N2);
+const void *vspec_pick_kernel_colgrp16_bands(int N2);
 cudaError_t vspec_colgrp4_debug_flags(unsigned *flags, bool clear);
 cudaError_t vspec_colgrp8_debug_flags(unsigned *flags, bool clear);
 cudaError_t vspec_colgrp16_debug_flags(unsigned *flags, bool clear);
@@ -204,6 +206,7 @@ struct vspec_plan {
     int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel (in twB's allocation)
     float2 *twBt = nullptr;      // its twiddles (in twB's allocation)
     bool pair = false;           // single-pol plans whose kernels run two spectra at once (scratch elements are pairs)
+    const void *kernelAb = nullptr;  // kernel A for interleaved sub-band tiles (else kernelA)
     int groupsA = 1;             // independent groups per kernel-A CTA (fir_colgrp_kernel)
     bool row_groups = false;     // kernel B is row2048_group_kernel
     bool row_batch = false;      // kernel B is row_batch_kernel (one-row transforms)
@@ -345,6 +348,19 @@ const void *pick_kernel_colgrp(int N2, int PT, int npol, size_t *smem, int *grou
     return PT == 4 ? vspec_pick_kernel_colgrp4(N2, npol, smem, groups)
          : PT == 8 ? vspec_pick_kernel_colgrp8(N2, npol, smem, groups)
                    : vspec_pick_kernel_colgrp16(N2, npol, smem, groups);
+}
+
+// ... for interleaved sub-band tiles (columns of at most 8 points, dual-pol).
+const void *pick_kernel_bands(int N2, int PT) {
+    using namespace vspec;
+    if (PT == 4) return vspec_pick_kernel_colgrp4_bands(N2);
+    if (PT == 16) return vspec_pick_kernel_colgrp16_bands(N2);
+    switch (N2) {
+        case 2: return (const void *)fir_colreg_kernel<2, 2, true>;
+        case 4: return (const void *)fir_colreg_kernel<4, 4, true>;
+        case 8: return (const void *)fir_colreg_kernel<8, 8, true>;
+    }
+    return nullptr;
 }
 
 // Kernel-A CTAs of a launch of `items` (tile, spectrum) items: at most nA, no
@@ -894,6 +910,7 @@ vspec_status build_plan(vspec_plan *p) {
     if (colreg) {
         p->kernelA = colreg;
         p->formA = p->pair ? "general-paired" : PT == 4 ? "colreg4" : PT == 16 ? "colreg16" : "colreg";
+        if (p->npol == 2) p->kernelAb = pick_kernel_bands(N2, PT);
     }
     // tensor-core plans with 2048-point rows and N2 = 16, 32, 64:
     //  - VSPEC_PLAN_TENSOR_INT8 (PFB of at most 8 taps, or direct): pre-filter
@@ -1068,6 +1085,7 @@ vspec_status build_plan(vspec_plan *p) {
         p->ring_grid = p->num_sms * occ;
     }
     VSPEC_CUDA(raise_smem_cap(p->kernelA, p->smemA));
+    if (p->kernelAb) VSPEC_CUDA(raise_smem_cap(p->kernelAb, p->smemA));
     VSPEC_CUDA(raise_smem_cap(p->kernelB, p->smemB));
     VSPEC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->occA, p->kernelA, p->TA, p->smemA));
     VSPEC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->occB, p->kernelB, p->TB, p->smemB));
@@ -1608,7 +1626,7 @@ static bool bands_fit(const vspec_plan *p, int nsub) {
 // chunk. With a power-of-two nsub a kernel-A tile is C consecutive words of
 // the interleaved rows (C / nsub columns of every band), staged with 16-byte
 // copies like plain input (8 x 4096 channels, 501 spectra: 548 -> 179 us with
-// one launch set for all bands; 8 x 32768, 125 spectra: kernel A 333 -> 223
+// one launch set for all bands, 143 us now with columns stored in band order; 8 x 32768, 125 spectra: kernel A 333 -> 223
 // us). Otherwise, and where more than two bands would leave a band fewer than
 // kSbTileCols columns of a tile (its scratch runs are then a sector or less:
 // kernel A at 8 x 65536 421 us gathered, 521 us interleaved; with two bands
@@ -1651,7 +1669,8 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
         ca.sc = sc;
         void *argsA[] = {&ca};
         const int ga = grid_a(nA, p->groupsA, ca.G, (long long)ca.tiles * sc);
-        vspec_status r = launch(p, 0, sc * nsub, p->kernelA, dim3(ga), dim3(p->TA), argsA, p->smemA, st);
+        const void *ka = ca.lsub && p->kernelAb ? p->kernelAb : p->kernelA;
+        vspec_status r = launch(p, 0, sc * nsub, ka, dim3(ga), dim3(p->TA), argsA, p->smemA, st);
         if (r != VSPEC_OK) return r;
         cb.s0 = s0;
         cb.sc = sc;

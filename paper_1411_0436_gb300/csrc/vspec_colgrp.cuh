@@ -60,7 +60,7 @@ struct ColGrp {
     static_assert(NCF <= 32 && 2 * NC * NT <= 32, "a thread's tensor-memory columns");
 };
 
-template <int N2_, int PT_, int GROUPS_, int NPOL>
+template <int N2_, int PT_, int GROUPS_, int NPOL, bool BANDS = false>
 __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constant__ ColParams p) {
     pdl_trigger();
     using G = ColGrp<N2_, PT_, GROUPS_>;
@@ -112,6 +112,10 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
         const int w0 = x * C;  // first column (or word) of the tile
         auto column = [&](int c) { return (w0 + c) >> p.lsub; };
         auto zcol = [&](int c) { return (p.lsub ? (size_t)((w0 + c) & (p.nsub - 1)) * p.N : 0) + column(c); };
+        // BANDS: interleaved tiles, columns transformed and stored in band order (BandOrder)
+        static_assert(!BANDS || G::kOnePass, "whole columns");
+        const BandOrder bo{p.nsub, p.lsub, p.lC - p.lsub};
+        auto outcol = [&](int c) { return BANDS ? (w0 >> p.lsub) + bo.out_col(c) : column(c); };
 
         // Ring slot (fr - first) mod RING holds absolute frame fr, first the
         // oldest frame of the run's first spectrum (frames before the input are
@@ -187,7 +191,7 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                 const int e = t + TG * i, c = e % C, row0 = G::kOnePass ? 0 : (e / C) % R1 * R2;
 #pragma unroll
                 for (int q = 0; q < G::NT; q++) {
-                    const float2 w = __ldg(p.twZ + (size_t)(row0 + q) * p.N1 + column(c));
+                    const float2 w = __ldg(p.twZ + (size_t)(row0 + q) * p.N1 + outcol(c));
                     v[2 * (i * G::NT + q)] = __float_as_uint(w.x);
                     v[2 * (i * G::NT + q) + 1] = __float_as_uint(w.y);
                 }
@@ -239,7 +243,7 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                     for (int u = 0; u < G::UB; u++) {
                         if (ub + u < nb) {
                             if (NPOL == 1 && p.half + s + ub + u >= p.nreal) y[u].re.y = y[u].im.y = 0.f;
-                            data[(ub + u) * SS + G::pad(pt)] = y[u];
+                            data[(ub + u) * SS + (BANDS ? pt / C * C + bo.of_word(pt % C) : G::pad(pt))] = y[u];
                         }
                     }
                 }
@@ -260,11 +264,12 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                     const int e = t + TG * k, c = e % C, sb = e / C;
                     if (sb < nb) {
                         P2 v[N2];
+                        const int rd = BANDS ? bo.of_out(c) : c;
 #pragma unroll
-                        for (int q = 0; q < N2; q++) v[q] = data[sb * SS + q * C + c];
+                        for (int q = 0; q < N2; q++) v[q] = data[sb * SS + q * C + rd];
                         Dft<N2>::run(v);
-                        P2 *z = Zc + (size_t)(s + sb) * zs + zcol(c);
-                        if (!dbg_ok(s + sb < p.sc && column(c) < p.N1, kDbgScratch)) continue;
+                        P2 *z = Zc + (size_t)(s + sb) * zs + (BANDS ? (size_t)bo.out_band(c) * p.N + outcol(c) : zcol(c));
+                        if (!dbg_ok(s + sb < p.sc && outcol(c) < p.N1, kDbgScratch)) continue;
                         z[0] = v[0];
 #pragma unroll
                         for (int q = 1; q < N2; q++) z[(size_t)q * p.N1] = cmul(v[q], twiddle(k % G::NC * N2 + q));

@@ -34,6 +34,16 @@ template <int PT> const void *pick_colgrp(int N2, int npol, size_t *smem, int *g
     return nullptr;
 }
 
+// ... for interleaved sub-band tiles, dual-pol, of at most 8-point columns.
+template <int PT> const void *pick_colgrp_bands(int N2) {
+    switch (N2) {
+        case 2: return (const void *)fir_colgrp_kernel<2, PT, colgrp_groups<2, PT>(), 2, true>;
+        case 4: return (const void *)fir_colgrp_kernel<4, PT, colgrp_groups<4, PT>(), 2, true>;
+        case 8: return (const void *)fir_colgrp_kernel<8, PT, colgrp_groups<8, PT>(), 2, true>;
+    }
+    return nullptr;
+}
+
 // This translation unit's bounds-check status word (debug builds).
 static inline cudaError_t colgrp_debug_flags(unsigned *flags, bool clear) {
 #ifdef VSPEC_DEBUG

@@ -504,6 +504,27 @@ __global__ void __launch_bounds__(512) fir_colfft_kernel(const __grid_constant__
     }
 }
 
+// Interleaved sub-band tiles (ColParams::lsub) of whole columns: the pre-filter
+// runs over a tile's words in input order (a column's bands side by side), the
+// columns and their stores in band order, c' = band Cb + column with Cb = C / nsub,
+// so that a warp stores runs of a band's columns and not a few columns of every
+// band. In between, column c' of a row is at band Cb + (column ^ f(band)), where 8
+// consecutive words, and 8 consecutive c', are in different banks. Cb >= 4. (8 x
+// 4096 channels, 501 spectra, GB300: kernel A 104 us with 64-byte runs, 72 us. An
+// instance of its own: in the plain kernels the index arithmetic costs 1.5%. Not
+// for 16-point columns: at most 4 to 8 columns of a band, 862 -> 909 us.)
+struct BandOrder {
+    int nsub, lsub, lcb;  // bands, their log2, log2 Cb
+    __device__ __forceinline__ int place(int band, int col) const {
+        const int f = lcb >= 3 ? (band << (3 - min(lsub, 3))) & 7 : ((band >> 1) << (2 - min(max(lsub, 1) - 1, 2))) & 3;
+        return (band << lcb) + (col ^ f);
+    }
+    __device__ __forceinline__ int out_band(int c) const { return c >> lcb; }
+    __device__ __forceinline__ int out_col(int c) const { return c & ((1 << lcb) - 1); }
+    __device__ __forceinline__ int of_word(int c) const { return place(c & (nsub - 1), c >> lsub); }
+    __device__ __forceinline__ int of_out(int c) const { return place(out_band(c), out_col(c)); }
+};
+
 // Kernel A, register-column form: dual-pol PFB of at most 8 taps in tiles of
 // 512 points (one per thread) with columns of N2 = 2 .. 128 points (nchan
 // 2^12 .. 2^18 with 2048-point rows, 2^19 with 4096-point rows). Plans launch it
@@ -557,7 +578,7 @@ struct ColReg {
 // Zc[s] (the chunk holds sc spectra). All PTS threads of the CTA take part;
 // the function ends with a barrier. twc: load the first-pass twiddles (they
 // stay in shared memory for later tiles of the same launch).
-template <int N2, int R1>
+template <int N2, int R1, bool BANDS = false>
 __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long long s0, int sc, int x, int s_beg,
                                             int s_end, unsigned char *smem_raw, bool load_twc, int band = 0) {
     using G = ColReg<N2, R1>;
@@ -573,15 +594,21 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
     const size_t zs = p.zstride > 0 ? (size_t)p.zstride : (size_t)p.N;  // scratch spectrum stride
     // this thread's column (its points and butterflies all have c = t mod C) and band
     const int w0 = x * C, n1t = (w0 + t % C) >> p.lsub;
+    // BANDS: this thread's point and column in band order (BandOrder)
+    static_assert(!BANDS || G::kOnePass, "whole columns");
+    const BandOrder bo{p.nsub, p.lsub, p.lC - p.lsub};
+    const int wr = BANDS ? t / C * C + bo.of_word(t % C) : t;
+    const int rd = BANDS ? bo.of_out(t % C) : t % C;
+    const int n1o = BANDS ? (w0 >> p.lsub) + bo.out_col(t % C) : n1t;
     if (p.lsub) {
         band = (w0 + t % C) & (p.nsub - 1);
-        Zc = reinterpret_cast<P2 *>(Zc) + (size_t)band * p.N;
+        Zc = reinterpret_cast<P2 *>(Zc) + (size_t)(BANDS ? bo.out_band(t % C) : band) * p.N;
     }
     // first-pass twiddles W_N2^(j q) (ordered before use by the loop's barriers)
     if (load_twc)
         for (int e = t; e < G::TWC; e += PTS) twc[e] = __ldg(p.twA + p.pass[0].off + e);
     {
-        tws[G::twi(t / C, t % C)] = __ldg(p.twZ + (size_t)(t / C) * p.N1 + n1t);  // W_N^(n1 k2), k2 = pos
+        tws[G::twi(t / C, t % C)] = __ldg(p.twZ + (size_t)(t / C) * p.N1 + n1o);  // W_N^(n1 k2), k2 = pos
 
         const long long n_pt = n1t + (long long)p.N1 * (t / C);
         // the tile's coefficients, read back for every batch so that their
@@ -652,7 +679,7 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
                     y.re = __ffma2_rn(cf2[k], wk.re, y.re);
                     y.im = __ffma2_rn(cf2[k], wk.im, y.im);
                 }
-                data[u * SS + G::pad(t)] = y;
+                data[u * SS + G::pad(wr)] = y;
             };
             if (nb == SPB) for_slots(fir_one, std::make_integer_sequence<int, SPB>{});
             else for_slots_below(fir_one, nb, std::make_integer_sequence<int, SPB>{});
@@ -665,10 +692,10 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
                     if (sb < nb) {
                         P2 v[N2];
 #pragma unroll
-                        for (int q = 0; q < N2; q++) v[q] = data[sb * SS + q * C + c];
+                        for (int q = 0; q < N2; q++) v[q] = data[sb * SS + q * C + rd];
                         Dft<N2>::run(v);
-                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + n1t;
-                        if (!dbg_ok(s_base + sb < sc && n1t < p.N1, kDbgScratch)) continue;
+                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + n1o;
+                        if (!dbg_ok(s_base + sb < sc && n1o < p.N1, kDbgScratch)) continue;
                         z[0] = v[0];
 #pragma unroll
                         for (int q = 1; q < N2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[G::twi(q, c)]);
@@ -718,7 +745,7 @@ __device__ __forceinline__ void colreg_tile(const ColParams &p, void *Zc, long l
     }
 }
 
-template <int N2, int R1 = N2>
+template <int N2, int R1 = N2, bool BANDS = false>
 __global__ void __launch_bounds__(512, 1) fir_colreg_kernel(const __grid_constant__ ColParams p) {
     pdl_trigger();
     extern __shared__ __align__(16) unsigned char smem_raw[];
@@ -735,7 +762,7 @@ __global__ void __launch_bounds__(512, 1) fir_colreg_kernel(const __grid_constan
             colreg_tile<N2, R1>(p, reinterpret_cast<P2 *>(p.Z) + (size_t)band * p.N, p.s0, p.sc, x / p.nsub, s_beg,
                                 s_end, smem_raw, first, band);
         } else {
-            colreg_tile<N2, R1>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.lsub ? 0 : p.band);
+            colreg_tile<N2, R1, BANDS>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.lsub ? 0 : p.band);
         }
         first = false;
     }
