@@ -1231,8 +1231,8 @@ vspec_status vspec_plan_create(vspec_plan **out, int nchan, int ntaps, int npol,
 // and hides its memory latency better, and beyond a per-size number of
 // spectra it is the faster path; below it the fused kernel's smaller fixed
 // cost wins. The thresholds come from measurements on GB300 (both paths timed
-// at 3 to 1200 spectra per call; cluster / two-kernel us: PFB 4096 channels 8
-// spectra 17.6 / 19.2, 16 19.3 / 18.2, 256 29.8 / 23.7; 8192 3 19.3 / 18.5, 256
+// at 3 to 1200 spectra per call; cluster / two-kernel us: PFB 4096 channels 3
+// spectra 18.5 / 16.4, 256 30.8 / 24.6; 8192 3 19.3 / 18.5, 256
 // 49.2 / 34.9; 16384 64 37.0 / 28.7; direct 4096 128 20.9 / 21.6, 192 23.6 / 21.7;
 // 8192 48 20.6 / 22.5, 64 23.9 / 22.5; 16384 24 22.1 / 24.6, 48 28.8 / 24.6; 32768
 // 8 20.6 / 22.5, 16 24.8 / 23.8). At 2048 channels the transform is one
@@ -1245,7 +1245,7 @@ vspec_status vspec_plan_create(vspec_plan **out, int nchan, int ntaps, int npol,
 // 0.62 of it with an 8-tap PFB, 0.70 in direct mode). With only a few idle
 // SMs the second path's fixed cost outweighs them.
 constexpr int kTwoKernelFrom[2][5] = {
-    {INT_MAX, 12, 0, 0, 0},    // PFB, nchan 2048 .. 32768
+    {INT_MAX, 0, 0, 0, 0},      // PFB, nchan 2048 .. 32768
     {INT_MAX, 150, 50, 30, 12}  // direct
 };
 constexpr double kAssistPerSmRate = 0.62;        // PFB

@@ -176,10 +176,22 @@ def _addr(x) -> Optional[int]:
     raise TypeError(f"cannot take the address of {type(x)}")
 
 
+_raw_stream = None  # torch's (current device) -> stream handle lookup, once CUDA is up
+
+
 def _stream(stream) -> Optional[int]:
     if stream is None:
+        # torch.cuda.current_stream() builds a Stream object for its handle: 3.1 us
+        # of a call's host time against 0.2 us for the lookup beneath it
+        global _raw_stream
+        if _raw_stream is not None:
+            return _raw_stream()
         import torch
-        return torch.cuda.current_stream().cuda_stream
+        handle = torch.cuda.current_stream().cuda_stream
+        get, dev = getattr(torch._C, "_cuda_getCurrentRawStream", None), getattr(torch._C, "_cuda_getDevice", None)
+        if get and dev:
+            _raw_stream = lambda: get(dev())
+        return handle
     if isinstance(stream, int):
         return stream
     return stream.cuda_stream
