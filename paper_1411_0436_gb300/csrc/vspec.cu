@@ -27,6 +27,7 @@
 #include "vspec_kernels_tcfir.cuh"
 #include "vspec_ring.cuh"
 #include "vspec_row2048.cuh"
+#include "vspec_row4096.cuh"
 #include "vspec_bp.cuh"
 #include "vspec_internal.h"
 
@@ -166,6 +167,7 @@ struct vspec_plan {
     int blocks_a = 0, blocks_b = 0;  // CTAs per kernel-A / kernel-B launch, 0: one wave
     bool fir_b = false;              // one-row transform: kernel B only, FIR in its first pass
     bool fold2048 = false;           // the fold runs reduce2048_kernel or its short form (2048-point rows, N2 >= 2)
+    bool fold4096 = false;           // the fold runs reduce2048_kernel's 4096-point form (N2 >= 64)
     bool gather = false;             // long PFB: kernel A reads the FIR taps from the input
     size_t smemA = 0, smemB = 0;
     std::vector<Pass> passA, passB;
@@ -203,12 +205,12 @@ struct vspec_plan {
     bool kahan = false;        // compensated accumulation at every level
     void *partial_comp = nullptr, *out_comp = nullptr;
     int *tc_status = nullptr;  // bounded-wait flag of the tensor-core or ring kernel
-    int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel (in twB's allocation)
+    int *row_status = nullptr;   // bounded-wait flag of row2048_group_kernel, row4096_group_kernel (in twB's allocation)
     float2 *twBt = nullptr;      // its twiddles (in twB's allocation)
     bool pair = false;           // single-pol plans whose kernels run two spectra at once (scratch elements are pairs)
     const void *kernelAb = nullptr;  // kernel A for interleaved sub-band tiles (else kernelA)
     int groupsA = 1;             // independent groups per kernel-A CTA (fir_colgrp_kernel)
-    bool row_groups = false;     // kernel B is row2048_group_kernel
+    bool row_groups = false;     // kernel B is row2048_group_kernel or row4096_group_kernel
     bool row_batch = false;      // kernel B is row_batch_kernel (one-row transforms)
     // persistent ring form (VSPEC_PLAN_RING): Z holds ringR slots of ringS
     // spectra, `partial` ring_sets partial-sum sets
@@ -521,6 +523,11 @@ vspec_status launch_fold(vspec_plan *p, int slots, float *d_accum, int spectra, 
                                      : (wide ? (const void *)reduce2048_kernel<1, 32, 1> : (const void *)reduce2048_kernel<1, 8, 4>);
         void *argsT[] = {&part, &span, &stride, (void *)&N, (void *)&N2, &ia, &outp};
         return launch(p, 2, spectra, k, dim3(N2 / 16 * 16 * (wide ? 4 : 16), nsub), dim3(wide ? 256 : 512), argsT, 0, st, 0, pdl);
+    }
+    if (p->fold4096) {  // (2^19 channels: 28.6 us in channel order)
+        const void *k = (const void *)vspec::reduce2048_kernel<2, 32, 1, 4096>;
+        void *argsT[] = {&part, &span, &stride, (void *)&N, (void *)&N2, &ia, &outp};
+        return launch(p, 2, spectra, k, dim3(N2 / 16 * 16 * 8, nsub), dim3(256), argsT, 0, st, 0, pdl);
     }
     void *argsR[] = {&part, &span, &stride, (void *)&N, (void *)&N1, (void *)&N2, &ia, &ib, &outp};
     return launch(p, 2, spectra, p->kernelR, dim3((N + 31) / 32, nsub), dim3(32, 8), argsR, 0, st, 0, pdl);
@@ -945,12 +952,12 @@ vspec_status build_plan(vspec_plan *p) {
     }
     if (p->fir_b) p->formA = "none";
     // dual-pol 4096-point rows without a pre-filter in kernel B, compensated
-    // sums or tensor-core rows: four radix-8 passes (row4096_kernel)
+    // sums or tensor-core rows: three radix-16 passes (row4096_group_kernel)
     const bool row4096 = N1 == 4096 && p->npol == 2 && !p->fir_b &&
                          !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8));
     const std::vector<int> rA = colblk ? std::vector<int>{8, N2 / 64, 8} : (tcfir || coltc) ? std::vector<int>{N2} : colreg ? r_colreg : coldir ? r_coldir
                                                                                : radix_list(e2, maxbitsA),
-                           rB = row4096 ? std::vector<int>{8, 8, 8, 8} : radix_list(e1);
+                           rB = row4096 ? std::vector<int>{16, 16, 16} : radix_list(e1);
     int twA_n = 0, twB_n = 0;
     p->passA = make_passes(N2, rA, &twA_n);
     p->passB = make_passes(N1, rB, &twB_n);
@@ -1047,13 +1054,14 @@ vspec_status build_plan(vspec_plan *p) {
             p->formB = N == 2048 ? "row2048-batched" : "general-batched";
         }
     }
-    // 4096-point rows (radix 8, 8, 8, 8): one spectrum per pass sequence,
-    // register accumulators
-    if (row4096 && !p->tc && p->RB == 1 && p->passB.size() == 4) {
-        p->kernelB = (const void *)vspec::row4096_kernel<false>;
-        p->TB = 512;
-        p->smemB = (size_t)vspec::kRow4096Stride * elem;
+    // 4096-point rows (radix 16, 16, 16)
+    if (row4096 && !p->tc && p->RB == 1 && p->passB.size() == 3) {
+        p->row_groups = true;
+        p->kernelB = (const void *)vspec::row4096_group_kernel;
+        p->TB = vspec::Row4096::THREADS;
+        p->smemB = vspec::Row4096::smem;
         p->formB = "row4096";
+        p->fold4096 = N2 >= 64;
     }
 
     // the persistent ring form: the register-column kernel A and the paired
