@@ -11,6 +11,10 @@
 // for a run of kRow2048Run spectra and 64 for the finished runs, added over the
 // groups in order once per segment.
 //
+// Pass-1 twiddles are in shared memory too: the row buffers leave L1 28 KB for
+// the 30 KB of them, and the warps waited most on those loads (whole call, 128
+// spectra: 763 us through L1, 740).
+//
 // Measured (GB300, 524288 channels, 128 spectra): 313 us against 382 us for four
 // radix-8 passes of one CTA-wide group with register sums. Bound, like the
 // 2048-point kernel, by the shared-memory data path.
@@ -24,8 +28,8 @@ struct Row4096 {
     static constexpr uint32_t ROW_BYTES = ROW * 16;
     static constexpr uint32_t TMEM_COLS = 512;  // 4 warps of a lane quarter x (64 run + 64 total)
     static constexpr int TW1 = 15 * 256, TW2 = 15 * 16;  // float2 entries of the [q-1][j] tables
-    // row buffers, pass-2 twiddles, barriers, the item last copied into each buffer, TMEM address, give-up flag
-    static constexpr size_t smem = (size_t)NBUF * ROW_BYTES + TW2 * 8 + NBUF * 12 + 12;
+    // row buffers, pass-1 and pass-2 twiddles, barriers, the item last copied into each buffer, TMEM address, give-up flag
+    static constexpr size_t smem = (size_t)NBUF * ROW_BYTES + (TW1 + TW2) * 8 + NBUF * 12 + 12;
     static_assert(smem <= 232448, "shared memory of one CTA");
 };
 
@@ -33,7 +37,8 @@ __global__ void __launch_bounds__(Row4096::THREADS, 1) row4096_group_kernel(cons
     using G = Row4096;
     extern __shared__ __align__(128) unsigned char smem_raw[];
     P2 *bufs = reinterpret_cast<P2 *>(smem_raw);                                           // [NBUF][4096]
-    float2 *tw2s = reinterpret_cast<float2 *>(smem_raw + (size_t)G::NBUF * G::ROW_BYTES);  // [15][16]
+    float2 *tw1s = reinterpret_cast<float2 *>(smem_raw + (size_t)G::NBUF * G::ROW_BYTES);  // [15][256]
+    float2 *tw2s = tw1s + G::TW1;                                                          // [15][16]
     uint64_t *full = reinterpret_cast<uint64_t *>(tw2s + G::TW2);                          // [NBUF]
     volatile int *copied = reinterpret_cast<volatile int *>(full + G::NBUF);               // [NBUF]
     uint32_t *tmem_slot = reinterpret_cast<uint32_t *>(const_cast<int *>(copied) + G::NBUF);
@@ -65,7 +70,7 @@ __global__ void __launch_bounds__(Row4096::THREADS, 1) row4096_group_kernel(cons
                      :: "r"(tc::smem_addr(tmem_slot)), "r"(G::TMEM_COLS) : "memory");
         asm volatile("tcgen05.relinquish_alloc_permit.cta_group::1.sync.aligned;" ::: "memory");
     }
-    for (int e = tid; e < G::TW2; e += G::THREADS) tw2s[e] = __ldg(p.twBt + G::TW1 + e);
+    for (int e = tid; e < G::TW1 + G::TW2; e += G::THREADS) tw1s[e] = __ldg(p.twBt + e);
     if (tid == 0) {
         *gave_up = 0;
         for (int b = 0; b < G::NBUF; b++) tc::mbar_init(full + b, 1);
@@ -85,7 +90,7 @@ __global__ void __launch_bounds__(Row4096::THREADS, 1) row4096_group_kernel(cons
     const int j = ht & 15;
     const int sw1 = ht ^ ((ht >> 4) & 7);  // pass 1: position ht + 256 q at sw1 + 256 q
     const int base2 = (ht >> 4) * 256;     // pass 2: position base2 + 16 q + j at base2 + 16 q + (j ^ (q & 7))
-    const float2 *tw1 = p.twBt + ht;       // W_4096^(ht q) at tw1[256 (q - 1)]
+    const float2 *tw1 = tw1s + ht;         // W_4096^(ht q) at tw1[256 (q - 1)]
 
     for (long long f = sp.lo; f < sp.hi;) {
         const int x = (int)(f / p.sc);  // row tile
@@ -114,7 +119,7 @@ __global__ void __launch_bounds__(Row4096::THREADS, 1) row4096_group_kernel(cons
             for (int i = 0; i < 16; i++) v[bitrev4(i)] = row[ht + 256 * bitrev4(i)];
             Dft<16>::run(v);
 #pragma unroll
-            for (int q = 1; q < 16; q++) v[q] = cmul(v[q], __ldg(tw1 + 256 * (q - 1)));
+            for (int q = 1; q < 16; q++) v[q] = cmul(v[q], tw1[256 * (q - 1)]);
             __syncwarp();  // the warp's lanes have read what they now overwrite
 #pragma unroll
             for (int q = 0; q < 16; q++) row[sw1 + 256 * q] = v[q];
