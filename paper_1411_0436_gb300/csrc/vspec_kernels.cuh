@@ -93,7 +93,7 @@ struct ColParams {
     // interleaved rows instead, word w being column w / nsub of band w mod nsub
     int nsub = 1, band = 0, lsub = 0;
     long long zstride = 0;  // scratch elements per spectrum (0: N)
-    // single-pol pairs (fir_colgrp_kernel, fir_coldir_kernel): pair s holds the
+    // single-pol pairs (fir_colgrp_kernel, fir_coldirgrp_kernel, fir_colblk_kernel): pair s holds the
     // chunk's spectra s and s + half, of which spectra below nreal exist
     int half = 0, nreal = 0;
 };
@@ -776,6 +776,7 @@ __global__ void __launch_bounds__(512, 1) fir_colreg_kernel(const __grid_constan
 // radix 16 then N2 / 16 (the plan's column pass list {16, N2/16}): the first
 // reads the staged bytes and writes fp32 to shared memory, the second writes
 // the chunk scratch. Every output is multiplied by W_N^(n1 k2) on its way out.
+// (The persistent batch runs this tile body; plans launch vspec_coldirgrp.cuh.)
 template <int N2>
 struct ColDir {
     static constexpr int PTS = 2048, C = PTS / N2, SPB = 4;
@@ -926,28 +927,6 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
             }
         }
         __syncthreads();  // the column passes are done with the twiddle tile and data
-    }
-}
-
-template <int N2>
-__global__ void __launch_bounds__(512) fir_coldir_kernel(const __grid_constant__ ColParams p) {
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    const TileSplit sp = tile_split(p.tiles, p.sc, p.G);
-    bool first = true;
-    for (long long f = sp.lo; f < sp.hi;) {
-        const long long base = f / p.sc * p.sc;  // first item of this super-tile
-        const int x = (int)(f / p.sc) * sp.G + sp.r;
-        const int s_beg = (int)(f - base);
-        const int s_end = (int)(min(sp.hi, base + p.sc) - base);
-        f = base + s_end;
-        if (p.band < 0 && !p.lsub) {  // every band in this launch: adjacent tiles are the bands of one column tile
-            const int band = x % p.nsub;
-            coldir_tile<N2>(p, reinterpret_cast<P2 *>(p.Z) + (size_t)band * p.N, p.s0, p.sc, x / p.nsub, s_beg, s_end,
-                            smem_raw, first, band);
-        } else {
-            coldir_tile<N2>(p, p.Z, p.s0, p.sc, x, s_beg, s_end, smem_raw, first, p.lsub ? 0 : p.band);
-        }
-        first = false;
     }
 }
 
