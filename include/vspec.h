@@ -175,22 +175,24 @@ VSPEC_API vspec_status vspec_plan_check(vspec_plan *plan);
  * that gives up (no GPU fault is involved in any of them).
  *
  * vspec_set_wait_limit sets, for every later launch in the process, how many
- * times a kernel polls before a bounded wait for its results gives up and
+ * times a kernel polls before a bounded wait for its results, or a row kernel
+ * (B=row2048, B=row4096) before a bounded wait for the copy of a row, gives up and
  * raises the plan's timeout flag (reported by vspec_plan_check or as
  * VSPEC_ERR_DEVICE_TIMEOUT by vspec_tc_dft16): polls >= 0 sets the limit (0
  * gives up at once), polls < 0 restores the default of 2^24 (a ring kernel
  * sleeps about 100 ns between polls; when one of its waits gives up, the
- * others return at once and the launch ends). The wait that
- * drains outstanding tensor-core work before a kernel frees its tensor
- * memory always keeps the default bound. Results computed under a wait that
- * gave up are incomplete and must be discarded.
+ * others return at once and the launch ends). The waits that
+ * drain outstanding tensor-core work before a kernel frees its tensor
+ * memory, and row copies before a CTA ends, always keep the default bound.
+ * Results computed under a wait that gave up are incomplete and must be discarded.
  * Errors: VSPEC_ERR_INVALID_ARG (polls above 2^32 - 1).
  *
  * vspec_plan_inject_timeout raises the plan's timeout flag from the host, as
  * if a device-side wait had expired; the next vspec_plan_check reports
  * VSPEC_ERR_DEVICE_TIMEOUT and clears it. Synchronous.
  * Errors: VSPEC_ERR_INVALID_ARG, VSPEC_ERR_UNSUPPORTED (a plan without
- * bounded device-side waits), VSPEC_ERR_CUDA.
+ * bounded waits for tensor-core or ring results; row copies' waits are made
+ * to give up with vspec_set_wait_limit(0)), VSPEC_ERR_CUDA.
  */
 VSPEC_API vspec_status vspec_set_wait_limit(long long polls);
 

@@ -1860,6 +1860,7 @@ static void make_params(const vspec_plan *p, const int8_t *d_in, int nspectra, v
     cb.twB = p->twB;
     cb.twBt = p->twBt;
     cb.wait_status = p->row_status;
+    cb.wait_limit = g_wait_limit.load();
     cb.N = p->N;
     cb.N1 = p->N1;
     cb.N2 = p->N2;
@@ -2335,7 +2336,7 @@ vspec_status vspec_set_wait_limit(long long polls) {
 vspec_status vspec_plan_inject_timeout(vspec_plan *plan) {
     if (!plan) return VSPEC_ERR_INVALID_ARG;
     if (!plan->tc_status) {
-        g_last_error = "this plan has no bounded device-side wait";
+        g_last_error = "this plan has no bounded wait for tensor-core or ring results";
         return VSPEC_ERR_UNSUPPORTED;
     }
     const int one = 1;

@@ -104,7 +104,8 @@ struct RowParams {
     void *partial_comp;  // Kahan compensation of `partial` (compensated plans only)
     const float2 *twB;   // per-pass twiddles of the length-N1 row DFTs
     const float2 *twBt;  // 2048-point rows: passes 1 and 2 in [q - 1][j] order (row2048_group_kernel)
-    int *wait_status;    // set to 1 if a bounded wait for a row's copy gave up (row2048_group_kernel)
+    int *wait_status;    // set to 1 if a bounded wait for a row's copy gave up (wait_row)
+    unsigned wait_limit; // polls of that wait
     int N, N1, N2, RB, npass;
     int lN1, lRB;        // log2 N1, log2 RB
     Pass pass[kMaxPasses];

@@ -60,6 +60,29 @@ __device__ __forceinline__ constexpr int bitrev4(int i) {
     return (i & 1) << 3 | (i & 2) << 1 | (i & 4) >> 1 | (i & 8) >> 3;
 }
 
+// Wait for the copy of item i into its buffer. The copy starts once the buffer's
+// previous item is done, which may be another group's: until `copied` shows it,
+// the barrier may be a phase behind, where the parity of the phase before it
+// reads as complete. Both waits are bounded by p.wait_limit (vspec_set_wait_limit);
+// one that gives up raises the plan's flag, and after it no row is copied any
+// more and the others do not wait.
+template <int NBUF>
+__device__ __forceinline__ void wait_row(const RowParams &p, uint64_t *full, const volatile int *copied,
+                                         volatile int *gave_up, int i) {
+    const int b = i % NBUF;
+    const uint32_t limit = *gave_up ? min(1u, p.wait_limit) : p.wait_limit;
+    bool started = copied[b] == i;
+    for (uint32_t it = 0; !started && it < limit; it++) started = copied[b] == i;
+    if (!started || !tc::mbar_wait(full + b, (i / NBUF) & 1, limit)) {
+        *gave_up = 1;
+        if (p.wait_status) atomicExch(p.wait_status, 1);
+    }
+}
+// After a wait that gave up: no copy of the CTA's n items may land once it has left.
+template <int NBUF> __device__ __forceinline__ void drain_rows(uint64_t *full, const volatile int *copied, int n) {
+    for (int b = 0; b < min(n, NBUF); b++) tc::mbar_wait(full + b, (copied[b] / NBUF) & 1);
+}
+
 // Scratch elements and sums: packed (X.re, Y.re, X.im, Y.im); split (X.re, X.im,
 // Y.re, Y.im), the tensor-core column kernel's order; or pairs, packed elements
 // whose halves are two spectra of a single polarisation (p.sc counts pairs):
@@ -137,18 +160,7 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
         for (int i = i0 + ((g - i0) & (G::GROUPS - 1)); i < i1; i += G::GROUPS) {
             const int b = i % G::NBUF;
             P2 *row = bufs + (size_t)b * 2048;
-            // The copy of item i starts once its buffer's previous item is done,
-            // which may be another group's: until `copied` shows it, the barrier
-            // may be a phase behind, where the parity of the phase before it
-            // reads as complete. Both waits are bounded; after one that gave up,
-            // the others do not wait.
-            const uint32_t limit = *gave_up ? 1u : tc::kSpinLimit;
-            bool started = copied[b] == i;
-            for (uint32_t it = 0; !started && it < limit; it++) started = copied[b] == i;
-            if (!started || !tc::mbar_wait(full + b, (i / G::NBUF) & 1, limit)) {
-                *gave_up = 1;
-                if (p.wait_status) atomicExch(p.wait_status, 1);
-            }
+            wait_row<G::NBUF>(p, full, copied, gave_up, i);
             __syncwarp();
             // pass 1: block length 2048, butterfly j = ht over positions ht + 128 q
             {
@@ -306,8 +318,7 @@ __global__ void __launch_bounds__(Row2048::THREADS, 1) row2048_group_kernel(cons
         }
     }
     pdl_trigger();
-    if (*gave_up && tid == 0)  // no copy may land after the CTA has left
-        for (int b = 0; b < min(n, G::NBUF); b++) tc::mbar_wait(full + b, (copied[b] / G::NBUF) & 1);
+    if (*gave_up && tid == 0) drain_rows<G::NBUF>(full, copied, n);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)

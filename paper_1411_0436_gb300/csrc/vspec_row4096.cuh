@@ -103,15 +103,7 @@ __global__ void __launch_bounds__(Row4096::THREADS, 1) row4096_group_kernel(cons
         for (int i = i0 + ((g - i0) & (G::GROUPS - 1)); i < i1; i += G::GROUPS) {
             const int b = i % G::NBUF;
             P2 *row = bufs + (size_t)b * G::ROW;
-            // (both waits as in row2048_group_kernel: bounded; after one that
-            // gave up, the others do not wait)
-            const uint32_t limit = *gave_up ? 1u : tc::kSpinLimit;
-            bool started = copied[b] == i;
-            for (uint32_t it = 0; !started && it < limit; it++) started = copied[b] == i;
-            if (!started || !tc::mbar_wait(full + b, (i / G::NBUF) & 1, limit)) {
-                *gave_up = 1;
-                if (p.wait_status) atomicExch(p.wait_status, 1);
-            }
+            wait_row<G::NBUF>(p, full, copied, gave_up, i);
             __syncwarp();
             P2 v[16];
             // pass 1: block length 4096, butterfly j = ht over positions ht + 256 q
@@ -217,8 +209,7 @@ __global__ void __launch_bounds__(Row4096::THREADS, 1) row4096_group_kernel(cons
         }
     }
     pdl_trigger();
-    if (*gave_up && tid == 0)  // no copy may land after the CTA has left
-        for (int b = 0; b < min(n, G::NBUF); b++) tc::mbar_wait(full + b, (copied[b] / G::NBUF) & 1);
+    if (*gave_up && tid == 0) drain_rows<G::NBUF>(full, copied, n);
     asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory");
     __syncthreads();
     if (warp == 0)
