@@ -791,16 +791,14 @@ vspec_status build_plan(vspec_plan *p) {
         grow();
     }
     if (p->req_n2) {  // a requested four-step split (vspec_plan_create_shaped)
+        // (a plan that takes the gather form keeps it: any column length the
+        // register window could hold leaves rows longer than 4096 points)
         const int n2 = p->req_n2;
-        const bool gather = pfb && N / n2 > 4096;
-        const int cap = gather ? 4096 / cmin : n2max();
-        if (!is_pow2(n2) || n2 > N || n2 > cap || N / n2 > 4096) {
+        if (!is_pow2(n2) || n2 > N || n2 > n2max() || N / n2 > 4096) {
             g_last_error = "requested column length outside what kernel A holds (N1 = nchan / col_len <= 4096)";
             return VSPEC_ERR_UNSUPPORTED;
         }
         N2 = n2;
-        p->gather = gather;
-        if (gather) PT = 1;
     }
     // pre-filtered plans whose rows come out at 2048 points (4096 at 2^19
     // dual-pol) with columns of at most 128 (single-pol 64: 128-point columns
