@@ -569,8 +569,9 @@ VSPEC_API vspec_status vspec_batch_bank_shape(const vspec_batch *batch, int bank
  * mode by timing both.
  *
  * vspec_batch_check synchronises and reports (once) whether a wait of the
- * persistent kernel gave up (VSPEC_ERR_DEVICE_TIMEOUT; the call's results are
- * incomplete). vspec_batch_inject_stall makes the next persistent execute
+ * persistent kernel, or in per-bank kernels a wait that vspec_plan_check of any
+ * bank's plan would report, gave up (VSPEC_ERR_DEVICE_TIMEOUT; the call's
+ * results are incomplete). vspec_batch_inject_stall makes the next persistent execute
  * start bank `bank`'s kernel-A done counter one below zero, so that its row
  * tickets' wait gives up (failure-path tests; no GPU fault is involved).
  */

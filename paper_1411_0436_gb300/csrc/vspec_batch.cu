@@ -426,12 +426,20 @@ vspec_status vspec_batch_get_persistent(const vspec_batch *batch, int *enabled) 
 
 vspec_status vspec_batch_check(vspec_batch *batch) {
     if (!batch) return VSPEC_ERR_INVALID_ARG;
-    if (!batch->bp_status) return VSPEC_OK;
-    int h = 0;
-    if (cudaMemcpy(&h, batch->bp_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return VSPEC_ERR_CUDA;
-    if (!h) return VSPEC_OK;
-    if (cudaMemset(batch->bp_status, 0, sizeof(int)) != cudaSuccess) return VSPEC_ERR_CUDA;
-    vspec_set_last_error("a bounded wait of the persistent multi-bank kernel gave up; results are incomplete");
+    bool expired = false;
+    if (batch->bp_status) {
+        int h = 0;
+        if (cudaMemcpy(&h, batch->bp_status, sizeof(int), cudaMemcpyDeviceToHost) != cudaSuccess) return VSPEC_ERR_CUDA;
+        if (h && cudaMemset(batch->bp_status, 0, sizeof(int)) != cudaSuccess) return VSPEC_ERR_CUDA;
+        expired = h != 0;
+    }
+    for (vspec_plan *p : batch->plans) {  // the banks' own kernels (every flag is read and cleared)
+        const vspec_status st = vspec_plan_check(p);
+        if (st != VSPEC_OK && st != VSPEC_ERR_DEVICE_TIMEOUT) return st;
+        expired |= st != VSPEC_OK;
+    }
+    if (!expired) return VSPEC_OK;
+    vspec_set_last_error("a bounded wait of the batch's kernels gave up; results are incomplete");
     return VSPEC_ERR_DEVICE_TIMEOUT;
 }
 

@@ -597,7 +597,7 @@ class Batch:
         return bool(v.value)
 
     def check(self) -> None:
-        """Raise if a bounded wait of the persistent kernel gave up (vspec_batch_check)."""
+        """Raise if a bounded wait of the persistent kernel or of a bank's kernels gave up (vspec_batch_check)."""
         st = load().vspec_batch_check(self.handle)
         if st != OK:
             raise VspecError(st, "vspec_batch_check")
