@@ -185,6 +185,8 @@ VSPEC_API vspec_status vspec_plan_check(vspec_plan *plan);
  * drain outstanding tensor-core work before a kernel frees its tensor
  * memory, and row copies before a CTA ends, always keep the default bound.
  * Results computed under a wait that gave up are incomplete and must be discarded.
+ * (A batch records its graph again when the limit changes; a graph that the
+ * caller captured keeps the limit of the capture.)
  * Errors: VSPEC_ERR_INVALID_ARG (polls above 2^32 - 1).
  *
  * vspec_plan_inject_timeout raises the plan's timeout flag from the host, as

@@ -2014,6 +2014,8 @@ static int bp_form(const vspec_plan *p0, const char **why) {
     return f;
 }
 
+unsigned vspec_wait_limit() { return g_wait_limit.load(); }
+
 void vspec_set_last_error(const char *what) { g_last_error = what ? what : ""; }
 
 vspec_status vspec_bp_supported(const vspec_plan *p, const char **why) {

@@ -39,6 +39,7 @@ struct vspec_batch {
     std::vector<const int8_t *> g_in;
     std::vector<int> g_ns;
     std::vector<float *> g_acc;
+    unsigned g_limit = 0;  // (and the wait limit of its kernels)
 };
 
 namespace {
@@ -66,6 +67,7 @@ vspec_status cuda_status(cudaError_t e) {
 vspec_status capture_graph(vspec_batch *b, const int8_t *const *d_in, const int *nspectra,
                            float *const *d_accum) {
     cudaGraph_t graph = nullptr;
+    const unsigned limit = vspec_wait_limit();
     cudaError_t e = cudaStreamBeginCapture(b->capture, cudaStreamCaptureModeThreadLocal);
     if (e != cudaSuccess) return VSPEC_ERR_CUDA;
     vspec_status st = VSPEC_OK;
@@ -101,12 +103,13 @@ vspec_status capture_graph(vspec_batch *b, const int8_t *const *d_in, const int 
     b->g_in.assign(d_in, d_in + b->nbanks);
     b->g_ns.assign(nspectra, nspectra + b->nbanks);
     b->g_acc.assign(d_accum, d_accum + b->nbanks);
+    b->g_limit = limit;
     return VSPEC_OK;
 }
 
 bool same_args(const vspec_batch *b, const int8_t *const *d_in, const int *nspectra,
                float *const *d_accum) {
-    if (!b->exec) return false;
+    if (!b->exec || b->g_limit != vspec_wait_limit()) return false;
     for (int i = 0; i < b->nbanks; i++)
         if (b->g_in[i] != d_in[i] || b->g_ns[i] != nspectra[i] || b->g_acc[i] != d_accum[i]) return false;
     return true;

@@ -15,5 +15,7 @@ vspec_status vspec_bp_supported(const vspec_plan *p, const char **why);
 // tickets wait for a kernel-A ticket that never comes (failure tests).
 vspec_status vspec_bp_execute(vspec_plan *const *plans, int n, const int8_t *const *d_in, const int *nspectra,
                               float *const *d_accum, int *ctl, int *status, int stall_bank, cudaStream_t st);
+// The limit of vspec_set_wait_limit that launches take now.
+unsigned vspec_wait_limit();
 // Set the text vspec_last_error reports on this thread.
 void vspec_set_last_error(const char *what);

@@ -40,3 +40,30 @@ def test_batch_check_reports_a_banks_wait_once(oracle_mod):
         for b, x, a in zip(BANKS, xs, accs):
             o = oracle_mod.channelize(x, b.nchan, b.ntaps, b.npol, b.nspectra, b.mode, b.window)
             assert_close(a.cpu().numpy().astype(np.float64).reshape(o.shape), o, what=f"bank {b.nchan} after a timeout")
+
+
+def test_recorded_batch_follows_the_wait_limit():
+    """A batch called again on the same buffers takes the limit in force, in
+    either direction."""
+    from paper_1411_0436_gb300 import vspec
+    b = BANKS[1]
+    d_in = torch.from_numpy(workloads.generate(b, 60).view(np.uint8).reshape(-1)).cuda()
+    with vspec.Batch([(b.nchan, b.ntaps, b.npol, b.mode, b.window)]) as batch:
+        acc = torch.zeros(batch.out_floats(0), dtype=torch.float32, device="cuda")
+
+        def call():
+            batch.execute([d_in], [b.nspectra], [acc])
+            torch.cuda.synchronize()
+
+        call()
+        batch.check()
+        try:
+            vspec.vspec_set_wait_limit(0)
+            call()
+        finally:
+            vspec.vspec_set_wait_limit(-1)
+        with pytest.raises(vspec.VspecError) as e:
+            batch.check()
+        assert e.value.status == vspec.ERR_DEVICE_TIMEOUT
+        call()
+        batch.check()
