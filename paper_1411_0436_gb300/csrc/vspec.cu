@@ -160,6 +160,7 @@ struct vspec_plan {
     const char *formA = "general";   // kernel A's form (vspec_plan_describe)
     const char *formB = "general";   // kernel B's form
     int num_sms = 0, occA = 1, occB = 1;
+    int maxA = 1;                    // kernel-A CTAs per SM that tuning limits allow for
     int maxB = 1;                    // kernel-B CTAs per SM that tuning limits and partial-sum slots allow for
     int sc_max = 1;                  // spectra per chunk
     int sc_cap = 1, slots_cap = 1;   // largest chunk a tuning may ask for; slots allocated
@@ -1104,6 +1105,10 @@ vspec_status build_plan(vspec_plan *p) {
     p->sc_cap = (int)std::max<size_t>(1, kScratchCap / per_spec);
     p->sc_max = std::min({p->sc_cap, kMaxChunkSpectra, (int)std::max<size_t>(1, kScratchBudget / per_spec)});
     if (p->fir_b) p->sc_cap = p->sc_max = kMaxChunkSpectra;  // launch length only: no scratch
+    // (fir_coldirgrp_kernel runs one CTA per SM at every column length; stored
+    // tunings of dual-pol plans with columns of 2 to 8 points come from a kernel
+    // that ran two)
+    p->maxA = coldir && p->npol == 2 && N2 <= 8 ? std::max(2, p->occA) : p->occA;
     // partial-sum slots for the largest kernel-B launch a tuning may ask for
     // (row2048_group_kernel and row_batch_kernel run one CTA per SM, but keep
     // the limits of the kernels that run the other plans of their sizes)
@@ -1461,7 +1466,7 @@ vspec_status vspec_plan_get_tuning(const vspec_plan *plan, vspec_tuning *current
         cur.blocks_a = tk->blocks_a;
         cur.blocks_b = tk->blocks_b;
         lim.chunk_spectra = tk->sc_cap;
-        lim.blocks_a = kMaxWaves * tk->num_sms * tk->occA;
+        lim.blocks_a = kMaxWaves * tk->num_sms * tk->maxA;
         lim.blocks_b = kMaxWaves * tk->num_sms * tk->maxB;
     }
     if (plan->fused) {
