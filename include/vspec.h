@@ -135,7 +135,13 @@ VSPEC_API vspec_status vspec_plan_create_ex(vspec_plan **out, int nchan, int nta
  * FP32 tolerance. Errors: as vspec_plan_create_ex, and VSPEC_ERR_UNSUPPORTED
  * for a shape the kernels cannot hold (the reason in vspec_last_error).
  * vspec_plan_get_shape reports a plan's col_len and tile_cols (0 for a
- * one-pass fused plan without a two-kernel plan).
+ * one-pass fused plan without a two-kernel plan). Both handed back give the
+ * plan's own two-kernel form again, with three exceptions: dual-pol plans with
+ * A=colreg (a pre-filter of 5..8 taps) or A=coldir take the general kernel A
+ * for them; the narrow tiles of A=colreg at 2^18 and 2^19 channels and the
+ * columns of one-row transforms are refused. Any other shape runs the general
+ * or the tap-gather kernel A, which
+ * is slower than the default's forms at most sizes.
  */
 VSPEC_API vspec_status vspec_plan_create_shaped(vspec_plan **out, int nchan, int ntaps, int npol,
                                                 vspec_mode mode, vspec_window window, unsigned flags,

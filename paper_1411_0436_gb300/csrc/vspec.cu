@@ -765,7 +765,54 @@ vspec_status build_fused_plan(vspec_plan *p) {
     return VSPEC_OK;
 }
 
+// Column length of the grouped kernel A, 0 for plans that do not take it:
+// pre-filtered plans whose rows come out at 2048 points (4096 at 2^19 dual-pol)
+// with columns of at most 128 (single-pol 64: 128-point columns would make
+// 8-byte tile rows, 292 us per 128 spectra of 262144 channels against 287 on
+// 4096-point rows); 512-point tiles.
+int colgrp_len(const vspec_plan *p) {
+    if (p->mode != VSPEC_PFB || p->N <= kRowElems ||
+        (p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)) ||
+        (p->npol == 1 && (p->flags & VSPEC_PLAN_KAHAN)))
+        return 0;
+    const int n2 = std::min(128, p->N / kRowElems), n1 = p->N / n2;
+    return (n1 == kRowElems && (p->npol == 2 || n2 <= 64)) || (p->npol == 2 && n1 == 2 * kRowElems) ? n2 : 0;
+}
+
+// ... of the blocked kernel A (2048-point rows and tiles): the longest
+// transforms (2^20 channels; single-pol pre-filters from 2^18 on, whose grouped
+// kernel would have 8-byte tile rows).
+int colblk_len(const vspec_plan *p, const void **kernel, size_t *smem) {
+    const bool pfb = p->mode == VSPEC_PFB;
+    *kernel = nullptr;
+    if ((p->N == 1 << 20 || (p->npol == 1 && pfb && p->N >= 1 << 18)) &&
+        (p->npol == 2 || !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR))))
+        *kernel = vspec_pick_kernel_colblk(p->N / kRowElems, p->npol, p->P, smem);
+    return *kernel ? p->N / kRowElems : 0;
+}
+
+// Whether the requested split and tile are those of the plan's own default form
+// (vspec_plan_get_shape), where that form's tiles are not the general kernel's:
+// such a request is the default plan. (The 8-tap dual-pol columns' shape stays
+// what it was: the general kernel, or refused where its tiles are narrower.)
+bool requests_own_shape(const vspec_plan *p) {
+    const void *k;
+    size_t smem;
+    int n2 = colblk_len(p, &k, &smem), pts = 2048;
+    if (!n2 && (p->npol == 1 || p->P <= 4 || p->P > 8)) {
+        n2 = colgrp_len(p);
+        pts = 512;
+    }
+    if (!n2 && p->npol == 1 && p->mode != VSPEC_PFB && p->N > kRowElems && p->N < 1 << 20 &&
+        !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR))) {
+        n2 = p->N / kRowElems;  // fir_coldirgrp_kernel
+        pts = 2048;
+    }
+    return n2 && p->req_n2 == n2 && p->req_cols == pts / n2;
+}
+
 vspec_status build_plan(vspec_plan *p) {
+    if (requests_own_shape(p)) p->req_n2 = p->req_cols = 0;
     const int N = p->N;
     const int e = ilog2(N);
     const bool pfb = p->mode == VSPEC_PFB;
@@ -801,34 +848,20 @@ vspec_status build_plan(vspec_plan *p) {
         }
         N2 = n2;
     }
-    // pre-filtered plans whose rows come out at 2048 points (4096 at 2^19
-    // dual-pol) with columns of at most 128 (single-pol 64: 128-point columns
-    // would make 8-byte tile rows, 292 us per 128 spectra of 262144 channels
-    // against 287 on 4096-point rows): kernel A in 512-point tiles
-    bool colgrp = false;
-    if (pfb && !p->req_n2 && !p->req_cols && N > kRowElems &&
-        !(p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)) &&
-        (p->npol == 2 || !(p->flags & VSPEC_PLAN_KAHAN))) {
-        const int n2 = std::min(128, N / kRowElems);
-        if ((N / n2 == kRowElems && (p->npol == 2 || n2 <= 64)) || (p->npol == 2 && N / n2 == 2 * kRowElems)) {
-            colgrp = true;
-            N2 = n2;
-            p->gather = false;
-            PT = p->P <= 4 ? 4 : p->P <= 8 ? 8 : 16;
-        }
+    const bool shaped = p->req_n2 || p->req_cols;
+    const int n2_grp = shaped ? 0 : colgrp_len(p);
+    const bool colgrp = n2_grp != 0;
+    if (colgrp) {
+        N2 = n2_grp;
+        p->gather = false;
+        PT = p->P <= 4 ? 4 : p->P <= 8 ? 8 : 16;
     }
-    // the longest transforms, with 2048-point rows: the blocked kernel A (2^20
-    // channels; single-pol pre-filters from 2^18 on, whose grouped kernel would
-    // have 8-byte tile rows)
     size_t smem_colblk = 0;
     const void *colblk = nullptr;
-    if (!p->req_n2 && !p->req_cols && (N == 1 << 20 || (p->npol == 1 && pfb && N >= 1 << 18)) &&
-        (p->npol == 2 || !(p->flags & (VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR)))) {
-        colblk = vspec_pick_kernel_colblk(N / kRowElems, p->npol, p->P, &smem_colblk);
-        if (colblk) {
-            N2 = N / kRowElems;
-            p->gather = false;
-        }
+    const int n2_blk = shaped ? 0 : colblk_len(p, &colblk, &smem_colblk);
+    if (colblk) {
+        N2 = n2_blk;
+        p->gather = false;
     }
     const int N1 = N / N2;
     if (N1 > 4096) {
