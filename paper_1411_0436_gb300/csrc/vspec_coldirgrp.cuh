@@ -98,7 +98,11 @@ __global__ void __launch_bounds__(512, 1) fir_coldirgrp_kernel(const __grid_cons
                 for (int i = 0; i < 4; i++) {
                     const int e = (t + TG * i) % (PTS / 8), y = (t + TG * i) / (PTS / 8);
                     const long long fy = fr + y * p.half;
-                    if (fy >= p.nframes) continue;  // the spectrum that an odd chunk lacks
+                    // (the second half's frame past the input is the spectrum that an odd chunk lacks)
+                    if (fy >= p.nframes) {
+                        if (!y) dbg_ok(false, kDbgInput);
+                        continue;
+                    }
                     const unsigned char *src = reinterpret_cast<const unsigned char *>(p.in) +
                                                (fy * p.N + (long long)p.N1 * (e / per_row) + w0 + e % per_row * 8) * 2;
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"

@@ -139,7 +139,10 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                                                (fr * p.N + (long long)p.N1 * (r / per_row) + w0) * 2 + r % per_row * CB;
                     unsigned char *dst = reinterpret_cast<unsigned char *>(ring) + (size_t)(y * RING + sl) * PTS * 2 + r * CB;
                     // (the second half's frames past the input belong to the spectrum an odd chunk lacks)
-                    if (fr >= p.nframes) continue;
+                    if (fr >= p.nframes) {
+                        if (!y) dbg_ok(false, kDbgInput);
+                        continue;
+                    }
                     if constexpr (CB == 16)
                         asm volatile("cp.async.cg.shared.global [%0], [%1], 16;" :: "r"(tc::smem_addr(dst)), "l"(src) : "memory");
                     else
