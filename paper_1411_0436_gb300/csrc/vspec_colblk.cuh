@@ -93,20 +93,20 @@ __global__ void __launch_bounds__(512, 1) fir_colblk_kernel(const __grid_constan
         const int w0 = x * C;  // first column
 
         // Ring slot (fr - first) mod RING holds absolute frame fr, first the
-        // oldest frame of the run's first spectrum (D leading taps have zero
-        // coefficients; frames before the input are clamped).
+        // oldest frame of the run's first spectrum (its D leading taps have zero
+        // coefficients: their frames are not copied).
         const long long first = p.s0 + s_beg - D;
         auto stage = [&](int rel, int cnt, int slot) {  // frames first + rel .. + cnt - 1 from ring slot `slot`
             auto frame = [&](int u, long long *fr, int *sl) {
                 *fr = first + rel + u;
-                if (*fr < 0) *fr = 0;
                 *sl = slot + u >= RING ? slot + u - RING : slot + u;
             };
             long long fr;
             int sl;
             if constexpr (NPOL == 1) {
                 constexpr int CB = C * 2 < 16 ? C * 2 : 16, per = PTS * 2 / CB, per_row = C * 2 / CB;
-                for (int i = t; i < 2 * cnt * per; i += G::THREADS) {
+                const int halves = p.half + s_beg < p.nreal ? 2 : 1;  // (a run of an odd chunk's last pair alone has one)
+                for (int i = t; i < halves * cnt * per; i += G::THREADS) {
                     const int y = i >= cnt * per, u = (i - y * cnt * per) / per, r = i % per;
                     frame(u, &fr, &sl);
                     if (y) fr += p.half;
@@ -137,7 +137,7 @@ __global__ void __launch_bounds__(512, 1) fir_colblk_kernel(const __grid_constan
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        stage(0, PT - 1 + min(SPB, s_end - s_beg), 0);
+        stage(D, PT - 1 - D + min(SPB, s_end - s_beg), D);
 
         // the run's constants: coefficient h of point k (tile element t + 512 k,
         // row n2 = that / C; in tensor memory at column 16 k + h); the twiddles of

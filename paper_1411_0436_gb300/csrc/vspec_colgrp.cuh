@@ -117,21 +117,22 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
         const BandOrder bo{p.nsub, p.lsub, p.lC - p.lsub};
         auto outcol = [&](int c) { return BANDS ? (w0 >> p.lsub) + bo.out_col(c) : column(c); };
 
-        // Ring slot (fr - first) mod RING holds absolute frame fr, first the
-        // oldest frame of the run's first spectrum (frames before the input are
-        // clamped: their taps have zero coefficients).
+        // Ring slot (fr - first) mod RING holds absolute frame fr, first the oldest
+        // frame of the run's first spectrum. Its D leading taps have zero
+        // coefficients: their frames are not copied (whatever bytes are in the slots
+        // are finite samples).
         const long long first = p.s0 + s_beg - D;
         auto stage = [&](int rel, int cnt, int slot) {  // frames first + rel .. + cnt - 1 from ring slot `slot`
             auto frame = [&](int u, long long *fr, int *sl) {
                 *fr = first + rel + u;
-                if (*fr < 0) *fr = 0;
                 *sl = slot + u >= RING ? slot + u - RING : slot + u;
             };
             long long fr;
             int sl;
             if constexpr (NPOL == 1) {
                 constexpr int CB = C * 2 < 16 ? C * 2 : 16, per = PTS * 2 / CB, per_row = C * 2 / CB;
-                for (int i = t; i < 2 * cnt * per; i += TG) {
+                const int halves = p.half + s_beg < p.nreal ? 2 : 1;  // (a run of an odd chunk's last pair alone has one)
+                for (int i = t; i < halves * cnt * per; i += TG) {
                     const int y = i >= cnt * per, u = (i - y * cnt * per) / per, r = i % per;
                     frame(u, &fr, &sl);
                     if (y) fr += p.half;
@@ -173,7 +174,7 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         // (the last run's readers of the ring are past its last barrier)
-        stage(0, PT - 1 + min(SPB, s_end - s_beg), 0);
+        stage(D, PT - 1 - D + min(SPB, s_end - s_beg), D);
 
         // the run's coefficients and four-step twiddles, into this thread's lane
         {
