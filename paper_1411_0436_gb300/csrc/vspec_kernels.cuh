@@ -176,6 +176,10 @@ struct SlotSpan {
 __device__ __forceinline__ int span_slots(const SlotSpan &w, int row) {
     if (w.n == 0) return w.all;
     const unsigned long long T = (unsigned long long)w.tiles * w.sc, x = row >> w.lrb;
+    if (T * w.n <= 0xffffffffu) {  // (a fold thread's two 64-bit divisions are most of a short fold)
+        const unsigned t = (unsigned)T, n = w.n, xs = (unsigned)x * w.sc;
+        return (int)(((xs + w.sc) * n - 1) / t - ((xs + 1) * n - 1) / t) + 1;
+    }
     const unsigned long long k_lo = ((x * w.sc + 1) * w.n - 1) / T, k_hi = ((x + 1) * w.sc * w.n - 1) / T;
     return (int)(k_hi - k_lo) + 1;
 }
