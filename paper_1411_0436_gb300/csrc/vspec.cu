@@ -192,6 +192,11 @@ struct vspec_plan {
     // kernel was at every length (PFB, us per call: 10 spectra 18.5 -> 16.4,
     // 1000 39 -> 27, 4096 103 -> 64; direct 4096 91 -> 47)
     vspec_plan *row_plan = nullptr;
+    // long transforms: calls of fewer than short_below spectra run this plan,
+    // the general or tap-gather kernel A (setup_short). Its own short_cap, if
+    // set, is its longest call; its coefficients are the owner's.
+    vspec_plan *short_plan = nullptr;
+    int short_below = 0, short_cap = 0;
     vspec_plan *owner = nullptr;  // the plan whose profiling records this plan's launches
     int assist_permille = 0;
     int two_kernel_from = INT_MAX;  // fused plans: calls with this many spectra use `assist` alone
@@ -580,9 +585,10 @@ void free_plan(vspec_plan *p) {
         cudaEventDestroy(p->ev_assist);
     }
     if (p->row_plan) free_plan(p->row_plan);
+    if (p->short_plan) free_plan(p->short_plan);
     for (cudaEvent_t e : p->event_pool) cudaEventDestroy(e);
     release_host_pipeline(p);
-    cudaFree(p->coef);
+    if (!p->short_cap) cudaFree(p->coef);
     cudaFree(p->twA);
     cudaFree(p->twB);
     cudaFree(p->twZ);
@@ -848,7 +854,7 @@ vspec_status build_plan(vspec_plan *p) {
         }
         N2 = n2;
     }
-    const bool shaped = p->req_n2 || p->req_cols;
+    const bool shaped = p->req_n2 || p->req_cols || p->short_cap;
     const int n2_grp = shaped ? 0 : colgrp_len(p);
     const bool colgrp = n2_grp != 0;
     if (colgrp) {
@@ -1138,6 +1144,7 @@ vspec_status build_plan(vspec_plan *p) {
     p->sc_cap = (int)std::max<size_t>(1, kScratchCap / per_spec);
     p->sc_max = std::min({p->sc_cap, kMaxChunkSpectra, (int)std::max<size_t>(1, kScratchBudget / per_spec)});
     if (p->fir_b) p->sc_cap = p->sc_max = kMaxChunkSpectra;  // launch length only: no scratch
+    if (p->short_cap) p->sc_cap = p->sc_max = std::min(p->sc_max, p->short_cap);
     // (fir_coldirgrp_kernel runs one CTA per SM at every column length; stored
     // tunings of dual-pol plans with columns of 2 to 8 points come from a kernel
     // that ran two)
@@ -1151,13 +1158,14 @@ vspec_status build_plan(vspec_plan *p) {
         VSPEC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->maxB, kernelB_limits, TB_limits, smem_limits));
         p->maxB = std::max(p->maxB, p->occB);
     }
-    p->slots_cap = slots_for(p, kMaxWaves * p->num_sms * p->maxB);
+    p->slots_cap = slots_for(p, p->short_cap ? p->num_sms * p->occB : kMaxWaves * p->num_sms * p->maxB);
 
     // device tables and scratch
     vspec_status st;
     size_t tot = 0;
     const int Lc = (pfb ? p->P : 1) * N;
-    if ((st = dev_alloc((void **)&p->coef, sizeof(float) * (size_t)Lc, &tot))) return st;
+    if (p->short_cap) p->coef = p->owner->coef;
+    else if ((st = dev_alloc((void **)&p->coef, sizeof(float) * (size_t)Lc, &tot))) return st;
     if ((st = dev_alloc((void **)&p->twA, sizeof(float2) * (size_t)std::max(1, twA_n), &tot))) return st;
     // with the row kernel's own twiddle order and wait flag after the table
     const bool own_tw = p->row_groups || p->row_batch;
@@ -1214,7 +1222,8 @@ vspec_status build_plan(vspec_plan *p) {
     if (ce == cudaSuccess) ce = cudaMemcpy(p->invA, invA.data(), sizeof(int) * N2, cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) ce = cudaMemcpy(p->invB, invB.data(), sizeof(int) * N1, cudaMemcpyHostToDevice);
     if (ce == cudaSuccess) {
-        vspec::gen_coef_kernel<<<(Lc + 255) / 256, 256, 0, s0>>>(p->coef, N, Lc, pfb ? 1 : 0, p->window);
+        if (!p->short_cap)
+            vspec::gen_coef_kernel<<<(Lc + 255) / 256, 256, 0, s0>>>(p->coef, N, Lc, pfb ? 1 : 0, p->window);
         for (const Pass &ps : p->passA)
             if (ps.m * (ps.r - 1) > 0)
                 vspec::gen_pass_tw_kernel<<<(ps.m * (ps.r - 1) + 255) / 256, 256, 0, s0>>>(p->twA, ps);
@@ -1331,6 +1340,50 @@ static vspec_status setup_assist(vspec_plan *p) {
     return VSPEC_OK;
 }
 
+// Short calls of the longest pre-filters. The grouped and blocked kernels start
+// a run (a tile's constants and P - 1 leading frames) for every tile of 512 or
+// 2048 points, and a call of one to three spectra is nothing but run starts; the
+// general and tap-gather kernels, with tiles of 4096 points and taps read spectrum
+// by spectrum, are faster there. Whole calls, GB300, us, grouped or blocked /
+// gather: 2^19 dual-pol 9 taps 1 spectrum 60 / 31, 3 spectra 90 / 69, 4 spectra 96 /
+// 82 (5: 103 / 98), 16 taps 3 spectra 111 / 106, 4 spectra 113 / 129; single-pol 8
+// taps 1 spectrum 33 / 25, 3 spectra 49 / 45, 4 spectra 51 / 51; 2^20 single-pol 8
+// taps 1 spectrum 97 / 78, 3 spectra 131 / 124, 4 spectra 133 / 143, 6 taps 1
+// spectrum 81 / 74, 2 spectra 93 / 98; dual-pol 16 taps 1 spectrum 130 / 113, 2
+// spectra 139 / 177.
+static int short_calls(const vspec_plan *p) {
+    if (p->fused || p->mode != VSPEC_PFB || p->req_n2 || p->req_cols ||
+        (p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)))
+        return 0;
+    if (p->N == 1 << 19) return p->npol == 1 || p->P > 8 ? 4 : 0;
+    if (p->N != 1 << 20) return 0;
+    if (p->npol == 2) return p->P > 8 ? 2 : 0;
+    return p->P > 8 || p->P < 6 ? 0 : p->P == 6 ? 2 : 4;  // (more than 8 taps: the gather form itself)
+}
+static vspec_status setup_short(vspec_plan *p) {
+    const int below = short_calls(p);
+    if (!below) return VSPEC_OK;
+    vspec_plan *q = new (std::nothrow) vspec_plan();
+    if (!q) return VSPEC_ERR_OOM;
+    q->N = p->N;
+    q->P = p->P;
+    q->npol = p->npol;
+    q->mode = p->mode;
+    q->window = p->window;
+    q->flags = p->flags;
+    q->owner = p;
+    q->short_cap = below - 1;
+    const vspec_status st = build_plan(q);
+    if (st != VSPEC_OK) {
+        free_plan(q);
+        return st == VSPEC_ERR_OOM ? VSPEC_OK : st;  // without it every call runs the plan's own kernels
+    }
+    p->short_plan = q;
+    p->short_below = below;
+    p->scratch_bytes += q->scratch_bytes;
+    return VSPEC_OK;
+}
+
 vspec_status vspec_plan_create_ex(vspec_plan **out, int nchan, int ntaps, int npol, vspec_mode mode,
                                   vspec_window window, unsigned flags) {
     return vspec_plan_create_shaped(out, nchan, ntaps, npol, mode, window, flags, 0, 0);
@@ -1380,6 +1433,7 @@ vspec_status vspec_plan_create_shaped(vspec_plan **out, int nchan, int ntaps, in
     if (flags & VSPEC_PLAN_RING) p->flags |= VSPEC_PLAN_TWO_KERNEL;  // the ring runs kernels A and B
     vspec_status st = build_plan(p);
     if (st == VSPEC_OK && p->fused) st = setup_assist(p);
+    if (st == VSPEC_OK) st = setup_short(p);
     if (st != VSPEC_OK) {
         free_plan(p);
         return st;
@@ -2159,6 +2213,9 @@ extern "C" {
 static vspec_status execute_one(vspec_plan *p, const int8_t *d_in, int nspectra, float *d_accum,
                                 cudaStream_t st) {
     if (p->ring) return run_ring(p, d_in, nspectra, d_accum, st);
+    // (a plan tuned to its own launch shape keeps it)
+    if (nspectra < p->short_below && p->blocks_a == 0 && p->blocks_b == 0 && nspectra <= p->sc_max)
+        return run_two_kernel(p->short_plan, d_in, nspectra, d_accum, st, nullptr);
     if (!p->fused) return run_two_kernel(p, d_in, nspectra, d_accum, st, nullptr);
     if (p->row_plan) return run_two_kernel(p->row_plan, d_in, nspectra, d_accum, st, nullptr);
     if (p->assist && nspectra >= p->two_kernel_from)
@@ -2323,7 +2380,8 @@ vspec_status vspec_plan_set_host_mode(vspec_plan *plan, int mode, size_t chunk_b
 vspec_status vspec_plan_check(vspec_plan *plan) {
     if (!plan) return VSPEC_ERR_INVALID_ARG;
     bool expired = false;
-    for (int *word : {plan->tc_status, plan->row_status, plan->assist ? plan->assist->row_status : nullptr}) {
+    for (int *word : {plan->tc_status, plan->row_status, plan->assist ? plan->assist->row_status : nullptr,
+                      plan->short_plan ? plan->short_plan->row_status : nullptr}) {
         if (!word) continue;
         int h = 0;
         VSPEC_CUDA(cudaMemcpy(&h, word, sizeof(int), cudaMemcpyDeviceToHost));
