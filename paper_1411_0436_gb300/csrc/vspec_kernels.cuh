@@ -105,7 +105,6 @@ struct RowParams {
     const float2 *twB;   // per-pass twiddles of the length-N1 row DFTs
     const float2 *twBt;  // 2048-point rows: passes 1 and 2 in [q - 1][j] order (row2048_group_kernel)
     int *wait_status;    // set to 1 if a bounded wait for a row's copy gave up (wait_row)
-    unsigned wait_limit; // polls of that wait
     int N, N1, N2, RB, npass;
     int lN1, lRB;        // log2 N1, log2 RB
     Pass pass[kMaxPasses];
@@ -121,6 +120,7 @@ struct RowParams {
     int store;           // 1: every slot has exactly one writer this call, which stores (no zeroing)
     long long nframes;   // frames the call's input holds (bounds checks of debug builds)
     long long band_bytes;  // row_batch_kernel: input of band b (of `tiles`) at b * band_bytes
+    unsigned wait_limit;   // polls of the bounded wait for a row's copy
 };
 
 // ------------------------------------------------------ dependent launches --
