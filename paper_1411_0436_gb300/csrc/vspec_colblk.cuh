@@ -96,7 +96,7 @@ __global__ void __launch_bounds__(512, 1) fir_colblk_kernel(const __grid_constan
         // oldest frame of the run's first spectrum (its D leading taps have zero
         // coefficients: their frames are not copied).
         const long long first = p.s0 + s_beg - D;
-        auto stage = [&](int rel, int cnt, int slot) {  // frames first + rel .. + cnt - 1 from ring slot `slot`
+        auto stage = [&](int rel, int cnt, int slot, int halves) {  // frames first + rel .. + cnt - 1 from ring slot `slot`
             auto frame = [&](int u, long long *fr, int *sl) {
                 *fr = first + rel + u;
                 *sl = slot + u >= RING ? slot + u - RING : slot + u;
@@ -105,7 +105,6 @@ __global__ void __launch_bounds__(512, 1) fir_colblk_kernel(const __grid_constan
             int sl;
             if constexpr (NPOL == 1) {
                 constexpr int CB = C * 2 < 16 ? C * 2 : 16, per = PTS * 2 / CB, per_row = C * 2 / CB;
-                const int halves = p.half + s_beg < p.nreal ? 2 : 1;  // (a run of an odd chunk's last pair alone has one)
                 for (int i = t; i < halves * cnt * per; i += G::THREADS) {
                     const int y = i >= cnt * per, u = (i - y * cnt * per) / per, r = i % per;
                     frame(u, &fr, &sl);
@@ -137,7 +136,8 @@ __global__ void __launch_bounds__(512, 1) fir_colblk_kernel(const __grid_constan
             }
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
-        stage(D, PT - 1 - D + min(SPB, s_end - s_beg), D);
+        // (a run of an odd chunk's last pair alone has one spectrum per pair)
+        stage(D, PT - 1 - D + min(SPB, s_end - s_beg), D, NPOL == 1 && p.half + s_beg >= p.nreal ? 1 : 2);
 
         // the run's constants: coefficient h of point k (tile element t + 512 k,
         // row n2 = that / C; in tensor memory at column 16 k + h); the twiddles of
@@ -226,7 +226,7 @@ __global__ void __launch_bounds__(512, 1) fir_colblk_kernel(const __grid_constan
                 }
             }
             __syncthreads();  // the batch's outputs are in data; the ring's oldest frames are free
-            if (s + SPB < s_end) stage(s - s_beg + RING, min(SPB, s_end - s - SPB), r0);
+            if (s + SPB < s_end) stage(s - s_beg + RING, min(SPB, s_end - s - SPB), r0, 2);
             r0 += SPB;
             if (r0 >= RING) r0 -= RING;
             // pass 1: block length N2, butterfly j = e / C over rows j + M1 q

@@ -122,7 +122,7 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
         // coefficients: their frames are not copied (whatever bytes are in the slots
         // are finite samples).
         const long long first = p.s0 + s_beg - D;
-        auto stage = [&](int rel, int cnt, int slot) {  // frames first + rel .. + cnt - 1 from ring slot `slot`
+        auto stage = [&](int rel, int cnt, int slot, int halves) {  // frames first + rel .. + cnt - 1 from ring slot `slot`
             auto frame = [&](int u, long long *fr, int *sl) {
                 *fr = first + rel + u;
                 *sl = slot + u >= RING ? slot + u - RING : slot + u;
@@ -131,7 +131,6 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
             int sl;
             if constexpr (NPOL == 1) {
                 constexpr int CB = C * 2 < 16 ? C * 2 : 16, per = PTS * 2 / CB, per_row = C * 2 / CB;
-                const int halves = p.half + s_beg < p.nreal ? 2 : 1;  // (a run of an odd chunk's last pair alone has one)
                 for (int i = t; i < halves * cnt * per; i += TG) {
                     const int y = i >= cnt * per, u = (i - y * cnt * per) / per, r = i % per;
                     frame(u, &fr, &sl);
@@ -174,7 +173,8 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
             asm volatile("cp.async.commit_group;" ::: "memory");
         };
         // (the last run's readers of the ring are past its last barrier)
-        stage(D, PT - 1 - D + min(SPB, s_end - s_beg), D);
+        // (a run of an odd chunk's last pair alone has one spectrum per pair)
+        stage(D, PT - 1 - D + min(SPB, s_end - s_beg), D, NPOL == 1 && p.half + s_beg >= p.nreal ? 1 : 2);
 
         // the run's coefficients and four-step twiddles, into this thread's lane
         {
@@ -253,7 +253,7 @@ __global__ void __launch_bounds__(512, 1) fir_colgrp_kernel(const __grid_constan
                 }
             }
             bar();  // the batch's outputs are in data; its oldest frames are free
-            if (s + SPB < s_end) stage(s - s_beg + RING, min(SPB, s_end - s - SPB), r0);
+            if (s + SPB < s_end) stage(s - s_beg + RING, min(SPB, s_end - s - SPB), r0, 2);
             r0 += SPB;
             if (r0 >= RING) r0 -= RING;
             uint32_t tw[32];
