@@ -1060,12 +1060,12 @@ vspec_status build_plan(vspec_plan *p) {
                          : coltc ? (const void *)row2048_group_kernel<kRowSplit> : (const void *)row2048_group_kernel<kRowPacked>;
         else if (p->npol == 2 && coltc)
             p->kernelB = (const void *)row2048_kernel<2, true, false, true>;
-        else if (p->npol == 2)
-            p->kernelB = k ? (f ? (const void *)row2048_kernel<2, true, true> : (const void *)row2048_kernel<2, true, false>)
-                           : (const void *)row2048_kernel<2, false, true>;
+        else if (p->npol == 2)  // (uncompensated one-row transforms: row_batch_kernel, below)
+            p->kernelB = f ? (const void *)row2048_kernel<2, true, true> : (const void *)row2048_kernel<2, true, false>;
         else
-            p->kernelB = k ? (f ? (const void *)row2048_kernel<1, true, true> : (const void *)row2048_kernel<1, true, false>)
-                           : (f ? (const void *)row2048_kernel<1, false, true> : (const void *)row2048_kernel<1, false, false>);
+            p->kernelB = f   ? (const void *)row2048_kernel<1, true, true>
+                         : k ? (const void *)row2048_kernel<1, true, false>
+                             : (const void *)row2048_kernel<1, false, false>;
         p->TB = p->row_groups ? Row2048::THREADS : 256;
         p->smemB = p->row_groups ? Row2048::smem : 2 * (size_t)kRow2048Stride * elem;
         p->formB = "row2048";
@@ -1153,7 +1153,9 @@ vspec_status build_plan(vspec_plan *p) {
     // (row2048_group_kernel and row_batch_kernel run one CTA per SM, but keep
     // the limits of the kernels that run the other plans of their sizes)
     p->maxB = p->row_groups ? std::max(2, p->occB) : p->occB;
-    if (p->row_batch || p->pair) {
+    if (p->row_batch && N == 2048) {
+        p->maxB = 2;  // the row kernel of two spectra at a time that these plans ran before
+    } else if (p->row_batch || p->pair) {
         VSPEC_CUDA(raise_smem_cap(kernelB_limits, smem_limits));
         VSPEC_CUDA(cudaOccupancyMaxActiveBlocksPerMultiprocessor(&p->maxB, kernelB_limits, TB_limits, smem_limits));
         p->maxB = std::max(p->maxB, p->occB);

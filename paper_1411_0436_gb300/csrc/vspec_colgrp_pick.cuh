@@ -14,12 +14,18 @@ template <int N2, int PT> constexpr int colgrp_groups() {
 }
 
 // Kernel A for columns of N2 points (2 .. 128) and PT taps at most, its dynamic
-// shared memory and groups per CTA.
+// shared memory and groups per CTA. (No plan asks for dual-pol 8-tap columns of
+// at most 16 points, which pick_kernel_colreg gives to the register window, nor
+// for single-pol 128-point columns, see colgrp_len: nullptr.)
 template <int N2, int PT> const void *colgrp_instance(int npol, size_t *smem, int *groups) {
     constexpr int GR = colgrp_groups<N2, PT>();
     *smem = ColGrp<N2, PT, GR>::smem;
     *groups = GR;
-    return npol == 2 ? (const void *)fir_colgrp_kernel<N2, PT, GR, 2> : (const void *)fir_colgrp_kernel<N2, PT, GR, 1>;
+    if constexpr (PT != 8 || N2 > 16)
+        if (npol == 2) return (const void *)fir_colgrp_kernel<N2, PT, GR, 2>;
+    if constexpr (N2 < 128)
+        if (npol == 1) return (const void *)fir_colgrp_kernel<N2, PT, GR, 1>;
+    return nullptr;
 }
 template <int PT> const void *pick_colgrp(int N2, int npol, size_t *smem, int *groups) {
     switch (N2) {
