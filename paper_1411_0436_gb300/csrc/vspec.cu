@@ -1299,9 +1299,9 @@ vspec_status vspec_plan_create(vspec_plan **out, int nchan, int ntaps, int npol,
 // path's per-SM rate against the clusters' SMs at the fused kernel's (about
 // 0.62 of it with an 8-tap PFB, 0.70 in direct mode). With only a few idle
 // SMs the second path's fixed cost outweighs them.
-constexpr int kTwoKernelFrom[2][5] = {
-    {INT_MAX, 0, 0, 0, 0},      // PFB, nchan 2048 .. 32768
-    {INT_MAX, 150, 50, 30, 12}  // direct
+constexpr int kTwoKernelFrom[2][4] = {
+    {0, 0, 0, 0},      // PFB, nchan 4096 .. 32768
+    {150, 50, 30, 12}  // direct
 };
 constexpr double kAssistPerSmRate = 0.62;        // PFB
 constexpr double kAssistPerSmRateDirect = 0.70;  // direct FFT
@@ -1322,7 +1322,7 @@ static vspec_status setup_assist(vspec_plan *p) {
         p->scratch_bytes += p->row_plan->scratch_bytes;
         return VSPEC_OK;
     }
-    p->two_kernel_from = (lg >= 0 && lg < 5) ? kTwoKernelFrom[p->mode == VSPEC_PFB ? 0 : 1][lg] : INT_MAX;
+    p->two_kernel_from = lg < 5 ? kTwoKernelFrom[p->mode == VSPEC_PFB ? 0 : 1][lg - 1] : INT_MAX;
     if (idle < kAssistMinSms && p->two_kernel_from == INT_MAX) return VSPEC_OK;
     vspec_plan *a = nullptr;
     vspec_status st = vspec_plan_create_ex(&a, p->N, p->mode == VSPEC_PFB ? p->P : 1, p->npol,

@@ -806,7 +806,7 @@ struct ColDir {
 // twiddles (they stay in shared memory for later tiles of the same launch).
 template <int N2>
 __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long long s0, int sc, int x, int s_beg,
-                                            int s_end, unsigned char *smem_raw, bool load_twc, int band = 0) {
+                                            int s_end, unsigned char *smem_raw, bool load_twc) {
     using G = ColDir<N2>;
     constexpr int PTS = G::PTS, C = G::C, SPB = G::SPB, R1 = G::R1, R2 = G::R2, M1 = G::M1;
     uint32_t *raw = reinterpret_cast<uint32_t *>(smem_raw);                        // [2][SPB][PTS]
@@ -816,10 +816,7 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
     float *wins = reinterpret_cast<float *>(twc + G::TWC);                         // [N2][C]
     const int t = threadIdx.x;
     const size_t zs = p.zstride > 0 ? (size_t)p.zstride : (size_t)p.N;  // scratch spectrum stride
-    // the tile's first word of a row; word w is column w / nsub of band w mod nsub (lsub > 0)
-    const int w0 = x * C;
-    auto column = [&](int c) { return (w0 + c) >> p.lsub; };
-    auto zcol = [&](int c) { return (p.lsub ? (size_t)((w0 + c) & (p.nsub - 1)) * p.N : 0) + column(c); };
+    const int n1_0 = x * C;  // first column
     if (load_twc)
         for (int e = t; e < G::TWC; e += 512) twc[e] = __ldg(p.twA + p.pass[0].off + e);
     // sample (pos e of the tile) of spectrum row rb, times the window value when there is one
@@ -833,34 +830,19 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
     };
     {
         for (int e = t; e < PTS; e += 512) {  // W_N^(n1 k2(pos)); window values h[n1 + N1 n2]
-            tws[e] = __ldg(p.twZ + (size_t)(e / C) * p.N1 + column(e % C));
-            if (p.win) wins[e] = __ldg(p.coef + (size_t)(e / C) * p.N1 + column(e % C));
+            tws[e] = __ldg(p.twZ + (size_t)(e / C) * p.N1 + n1_0 + e % C);
+            if (p.win) wins[e] = __ldg(p.coef + (size_t)(e / C) * p.N1 + n1_0 + e % C);
         }
-        // frames of SPB spectra into raw[buf], 16-byte copies (sub-band input:
-        // 4-byte copies of this band's samples, nsub words apart)
+        // frames of SPB spectra into raw[buf], 16-byte copies
         auto stage = [&](int sb, int buf) {
             const int nbb = min(SPB, s_end - sb);
-            if (p.nsub > 1 && !p.lsub) {
-                for (int e = t; e < nbb * PTS; e += 512) {
-                    const int u = e / PTS, r = e % PTS;  // r = n2 C + c
-                    const long long fr = s0 + sb + u;
-                    const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) +
-                                          (fr * p.N + w0 + (long long)p.N1 * (r / C) + r % C) * p.nsub + band;
-                    uint32_t *dst = raw + (buf * SPB + u) * PTS + r;
-                    if (dbg_ok(fr < p.nframes, kDbgInput))
-                        asm volatile("cp.async.ca.shared.global [%0], [%1], 4;"
-                                     :: "r"((uint32_t)__cvta_generic_to_shared(dst)), "l"(src) : "memory");
-                }
-                asm volatile("cp.async.commit_group;" ::: "memory");
-                return;
-            }
             constexpr int per_row = C / 4, per_frame = PTS / 4;
             for (int e = t; e < nbb * per_frame; e += 512) {
                 const int u = e / per_frame, r = e % per_frame;
                 const int n2 = r / per_row, ch = r % per_row;
                 const long long fr = s0 + sb + u;
                 const uint32_t *src = reinterpret_cast<const uint32_t *>(p.in) +
-                                      ((fr * p.N + (long long)p.N1 * n2) << p.lsub) + w0 + ch * 4;
+                                      fr * p.N + n1_0 + (long long)p.N1 * n2 + ch * 4;
                 uint32_t *dst = raw + (buf * SPB + u) * PTS + n2 * C + ch * 4;
                 if (dbg_ok(fr < p.nframes, kDbgInput))
                     asm volatile("cp.async.cg.shared.global [%0], [%1], 16;"
@@ -885,8 +867,8 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
 #pragma unroll
                         for (int q = 0; q < N2; q++) v[q] = sample(rb + sb * PTS, q * C + c);
                         Dft<N2>::run(v);
-                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + zcol(c);
-                        if (!dbg_ok(s_base + sb < sc && column(c) < p.N1, kDbgScratch)) continue;
+                        P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs + n1_0 + c;
+                        if (!dbg_ok(s_base + sb < sc && n1_0 + c < p.N1, kDbgScratch)) continue;
                         z[0] = v[0];
 #pragma unroll
                         for (int q = 1; q < N2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[q * C + c]);
@@ -923,8 +905,8 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
                         for (int q = 0; q < R2; q++) v[q] = d[q * C];
                         Dft<R2>::run(v);
                         P2 *z = reinterpret_cast<P2 *>(Zc) + (size_t)(s_base + sb) * zs +
-                                (size_t)(b * R2) * p.N1 + zcol(c);
-                        if (!dbg_ok(s_base + sb < sc && column(c) < p.N1, kDbgScratch)) continue;
+                                (size_t)(b * R2) * p.N1 + n1_0 + c;
+                        if (!dbg_ok(s_base + sb < sc && n1_0 + c < p.N1, kDbgScratch)) continue;
 #pragma unroll
                         for (int q = 0; q < R2; q++) z[(size_t)q * p.N1] = cmul(v[q], tws[(b * R2 + q) * C + c]);
                     }
