@@ -332,17 +332,28 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  * tests, e.g. "two-kernel N1=2048 N2=16 C=32 A=colreg B=row2048 chunk=2048".
  * Words:
  *   fused K=<cluster CTAs>   the one-pass cluster kernel, then " | " and the
- *                            two-kernel plan it switches to
+ *                            two-kernel plan it switches to at two_kernel_from
+ *                            spectra (by default 0 with a pre-filter: every
+ *                            call runs that plan)
  *   two-kernel               the general path
- *   A=colreg|coldir|general|gather|none   kernel A's form: register columns
- *                            (dual-pol PFB; colreg4, colreg16: up to 4, up to
- *                            16 taps), register columns (dual-pol direct), the
- *                            general kernel (general-paired: two single-pol
- *                            spectra at once), taps read from the
- *                            input (gather-blocked: columns of the longest
- *                            transforms, from frames staged in shared memory); none for one-row transforms
- *   B=row2048|general|tensor kernel B's form (-batched: the one-row kernel of
- *                            512, 1024 and 2048 channels)
+ *   A=<form>                 kernel A; compare the whole word, some are parts of others:
+ *     colreg                 dual-pol pre-filter of 5..8 taps: register window for columns of
+ *                            at most 16 points, the grouped kernel above
+ *     colreg4, colreg16      the grouped kernel for up to 4, for 9..16 taps
+ *     coldir                 dual-pol direct columns
+ *     general-paired         the grouped (pre-filter) or direct kernel on pairs of single-pol
+ *                            spectra (not the general kernel: the word is kept for callers
+ *                            that look for single-pol plans by it)
+ *     gather-blocked         the blocked kernel of the longest columns, from frames staged in
+ *                            shared memory
+ *     general, gather        the general kernel; its form that reads every tap from the input
+ *     tensor, tensor-int8    the tensor-core forms
+ *     none                   one-row transforms
+ *   B=<form>                 kernel B: row2048, row4096, tensor, general; row2048-batched and
+ *                            general-batched are the one-row kernel of 2048 and of 512 and
+ *                            1024 channels
+ *   | below <k> spectra      then the two-kernel plan that runs such calls (2^19 and 2^20
+ *                            channels)
  *   fir-in-B                 one-row transform: the FIR runs in kernel B
  *   kahan                    compensated accumulation
  * Writes at most len bytes including the terminating NUL (truncating).

@@ -1286,8 +1286,11 @@ vspec_status vspec_plan_create(vspec_plan **out, int nchan, int ntaps, int npol,
 // and hides its memory latency better, and beyond a per-size number of
 // spectra it is the faster path; below it the fused kernel's smaller fixed
 // cost wins. The thresholds come from measurements on GB300 (both paths timed
-// at 3 to 1200 spectra per call; cluster / two-kernel us: PFB 4096 channels 3
-// spectra 18.5 / 16.4, 256 30.8 / 24.6; 8192 3 19.3 / 18.5, 256
+// at 1 to 1200 spectra per call; cluster / two-kernel us: PFB 1 spectrum 4096
+// channels 14.6 / 12.4, 8192 14.6 / 12.6, 16384 15.0 / 12.6, 32768 25.8 / 14.0, 8
+// spectra 14.6 / 12.5, 16.5 / 14.3, 16.4 / 16.6, 29.4 / 18.6, 16 spectra of 16384
+// 20.6 / 18.7 (those back to back; what follows with the launch of one call before
+// it done); 4096 3 18.5 / 16.4, 256 30.8 / 24.6; 8192 3 19.3 / 18.5, 256
 // 49.2 / 34.9; 16384 64 37.0 / 28.7; direct 4096 128 20.9 / 21.6, 192 23.6 / 21.7;
 // 8192 48 20.6 / 22.5, 64 23.9 / 22.5; 16384 24 22.1 / 24.6, 48 28.8 / 24.6; 32768
 // 8 20.6 / 22.5, 16 24.8 / 23.8). At 2048 channels the transform is one
@@ -1538,6 +1541,8 @@ vspec_status vspec_plan_describe(const vspec_plan *plan, char *buf, size_t len) 
         if (plan->row_plan) d += " | " + two_kernel(plan->row_plan);
     } else {
         d = two_kernel(plan);
+        if (plan->short_plan)
+            d += " | below " + std::to_string(plan->short_below) + " spectra " + two_kernel(plan->short_plan);
     }
     const size_t n = std::min(len - 1, d.size());
     std::memcpy(buf, d.data(), n);

@@ -28,6 +28,7 @@ def test_short_calls_match_oracle_and_add_up(oracle_mod, n, p, npol, below):
         return oracle_mod.channelize(np.ascontiguousarray(part), n, p, npol, count, PFB, WIN_HANN)
 
     with Plan(n, p, npol, PFB, WIN_HANN) as plan:
+        assert f" | below {below} spectra two-kernel " in plan.describe() and " A=gather " in plan.describe()
         acc = torch.zeros(plan.out_floats, dtype=torch.float32, device="cuda")
 
         def spectrum():
