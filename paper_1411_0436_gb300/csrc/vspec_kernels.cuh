@@ -920,7 +920,10 @@ __device__ __forceinline__ void coldir_tile(const ColParams &p, void *Zc, long l
 // Kernel A for transforms too long for a register FIR window next to the
 // column tile (PFB with nchan above 2^18): every spectrum's P taps are read
 // straight from the input (the P frames a spectrum spans stay in L2 while
-// the block walks its consecutive spectra), the coefficients from L1/L2.
+// the block walks its consecutive spectra), the coefficients from L1/L2. Plans
+// launch it for single-pol 2^20 with more than 8 taps, for requested shapes and
+// for calls of one to three spectra (setup_short); the grouped and blocked
+// kernels have the rest.
 template <int NPOL, int PPT>
 __global__ void __launch_bounds__(512) fir_colfft_gather_kernel(const __grid_constant__ ColParams p) {
     pdl_trigger();
@@ -1279,9 +1282,10 @@ __global__ void __launch_bounds__(256, 2) rowfft_detect_kernel(const __grid_cons
 }
 
 // ------------------------------------------------------ kernel B, 2048 --
-// Single-polarisation, compensated and one-row plans, and the row bodies of
-// the persistent forms; other dual-pol plans run row2048_group_kernel
-// (vspec_row2048.cuh).
+// Compensated plans, single-polarisation plans without pairs (a requested
+// shape) and the row bodies of the persistent forms; the others run
+// row2048_group_kernel (vspec_row2048.cuh) or, with one row, row_batch_kernel
+// (vspec_rowbatch.cuh).
 // Rows of 2048 points (RB = 1; passes radix 16, 16, 8), two spectra at a
 // time. In the radix-16 passes (128 butterflies each) the block's halves
 // transform one spectrum each, synchronising on their own named barrier;

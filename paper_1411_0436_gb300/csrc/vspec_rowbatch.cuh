@@ -3,7 +3,8 @@
 // the int8 input, with nothing in between leaving the SM.
 //
 // One 512-thread CTA per SM takes a run of consecutive spectra in batches of
-// 8192 points (SPB spectra). Per batch:
+// 8192 points (SPB spectra; 4096 points at 2048 channels dual-pol with more than
+// 8 taps). Per batch:
 //  - the pre-filter: each thread forms its points' outputs of the whole batch
 //    from one walk over a ring of staged int8 frames, unpacking a sample once
 //    for all the outputs it is a tap of (PT - 1 + SPB unpacks for SPB outputs);
@@ -24,7 +25,7 @@
 // are the two halves of each pair. Both powers go to the same sum.
 //
 // What bounds it: about 104 bytes of shared-memory traffic and 113 FMA-pipe
-// slots per point, phase after phase (5 barriers per 8192 points); on short
+// slots per point, phase after phase (four barriers per batch); on short
 // calls its prologue (coefficients, PT - 1 leading frames) and latency.
 // Measured (GB300, whole calls, us): 1024 channels dual-pol 8 taps 2048 spectra
 // 66 -> 22.6, 4096 spectra 114 -> 35, direct 60 -> 29; single-pol 4096 spectra
