@@ -1754,7 +1754,8 @@ static vspec_status run_bands(vspec_plan *p, int nsub, const int8_t *d_in, int n
     const int slots = (int)(std::min<long long>(nB, (long long)tilesB * sc_full) / tilesB + 2);
     const int gb_full = (int)std::min<long long>(nB, (long long)tilesB * sc_full);
     const vspec::SlotSpan written{gb_full, tilesB, sc_full, 0, ilog2(p->RB)};
-    const bool store = nchunks == 1 && slots <= kFoldSlots;  // as in run_two_kernel
+    const bool store = nchunks == 1 && slots <= kFoldSlots &&
+                       vspec::span_fits(gb_full, tilesB, sc_full);  // as in run_two_kernel
     if (!store) VSPEC_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)slots * NV * sizeof(float4), st));
     vspec::ColParams ca;
     vspec::RowParams cb;
@@ -1991,8 +1992,9 @@ static vspec_status run_two_kernel(vspec_plan *p, const int8_t *d_in, int nspect
     // stores it, and the fold reads only the slots that were written, so nothing
     // needs zeroing (the memset cost 2 - 3 us of a 30 us call). One-row
     // transforms: block k writes slot k, and the fold reads those.
-    const bool store = !p->kahan && !p->tc && nchunks == 1 && (p->fir_b || slots <= kFoldSlots);
     const int gb_full = (int)std::min<long long>(nB, (long long)tilesB * rows(sc_full));
+    const bool store = !p->kahan && !p->tc && nchunks == 1 &&
+                       (p->fir_b || (slots <= kFoldSlots && vspec::span_fits(gb_full, tilesB, rows(sc_full))));
     const vspec::SlotSpan written{gb_full, tilesB, rows(sc_full), 0, ilog2(p->RB)};
     if (store && p->fir_b) slots = gb_full;
     if (!store) VSPEC_CUDA(cudaMemsetAsync(p->partial, 0, (size_t)slots * p->N * accel, st));

@@ -168,20 +168,17 @@ __device__ __forceinline__ int span_slot(int tiles, int sc, int x) {
 
 // Slots of row tile x that a launch of n blocks (at most one per item) wrote:
 // the blocks between those that hold the tile's first and last item, ranks 0 ..
-// .. n = 0: `all` slots (zeroed, or every one written).
+// .. n = 0: `all` slots (zeroed, or every one written). n tiles sc fits 32 bits (span_fits): a fold
+// thread's two 64-bit divisions were most of a short fold.
 struct SlotSpan {
     int n, tiles, sc, all;
     int lrb;  // log2 rows per tile
 };
+inline bool span_fits(long long n, long long tiles, long long sc) { return tiles * sc <= 0xffffffffll / n; }
 __device__ __forceinline__ int span_slots(const SlotSpan &w, int row) {
     if (w.n == 0) return w.all;
-    const unsigned long long T = (unsigned long long)w.tiles * w.sc, x = row >> w.lrb;
-    if (T * w.n <= 0xffffffffu) {  // (a fold thread's two 64-bit divisions are most of a short fold)
-        const unsigned t = (unsigned)T, n = w.n, xs = (unsigned)x * w.sc;
-        return (int)(((xs + w.sc) * n - 1) / t - ((xs + 1) * n - 1) / t) + 1;
-    }
-    const unsigned long long k_lo = ((x * w.sc + 1) * w.n - 1) / T, k_hi = ((x + 1) * w.sc * w.n - 1) / T;
-    return (int)(k_hi - k_lo) + 1;
+    const unsigned T = (unsigned)w.tiles * w.sc, n = w.n, xs = (unsigned)(row >> w.lrb) * w.sc;
+    return (int)(((xs + w.sc) * n - 1) / T - ((xs + 1) * n - 1) / T) + 1;
 }
 
 // Kernel A's split: blocks come in groups of G consecutive blocks that take
