@@ -352,8 +352,8 @@ VSPEC_API vspec_status vspec_plan_info(const vspec_plan *plan, size_t *scratch_b
  *   B=<form>                 kernel B: row2048, row4096, tensor, general; row2048-batched and
  *                            general-batched are the one-row kernel of 2048 and of 512 and
  *                            1024 channels
- *   | below <k> spectra      then the two-kernel plan that runs such calls (2^19 and 2^20
- *                            channels)
+ *   | spectra=<n>,<n>...     then the two-kernel plan that runs calls of so many spectra (2^19
+ *                            and 2^20 channels)
  *   fir-in-B                 one-row transform: the FIR runs in kernel B
  *   kahan                    compensated accumulation
  * Writes at most len bytes including the terminating NUL (truncating).

@@ -192,11 +192,12 @@ struct vspec_plan {
     // kernel was at every length (PFB, us per call: 10 spectra 18.5 -> 16.4,
     // 1000 39 -> 27, 4096 103 -> 64; direct 4096 91 -> 47)
     vspec_plan *row_plan = nullptr;
-    // long transforms: calls of fewer than short_below spectra run this plan,
-    // the general or tap-gather kernel A (setup_short). Its own short_cap, if
-    // set, is its longest call; its coefficients are the owner's.
+    // long transforms: calls of n spectra, bit n of short_counts set, run this
+    // plan, the general or tap-gather kernel A (setup_short). Its own short_cap,
+    // if set, is its longest call; its coefficients are the owner's.
     vspec_plan *short_plan = nullptr;
-    int short_below = 0, short_cap = 0;
+    unsigned short_counts = 0;
+    int short_cap = 0;
     vspec_plan *owner = nullptr;  // the plan whose profiling records this plan's launches
     int assist_permille = 0;
     int two_kernel_from = INT_MAX;  // fused plans: calls with this many spectra use `assist` alone
@@ -1352,22 +1353,24 @@ static vspec_status setup_assist(vspec_plan *p) {
 // by spectrum, are faster there. Whole calls, GB300, us, grouped or blocked /
 // gather: 2^19 dual-pol 9 taps 1 spectrum 60 / 31, 3 spectra 90 / 69, 4 spectra 96 /
 // 82 (5: 103 / 98), 16 taps 3 spectra 111 / 106, 4 spectra 113 / 129; single-pol 8
-// taps 1 spectrum 33 / 25, 3 spectra 49 / 45, 4 spectra 51 / 51; 2^20 single-pol 8
-// taps 1 spectrum 97 / 78, 3 spectra 131 / 124, 4 spectra 133 / 143, 6 taps 1
+// taps 1 spectrum 33 / 25, 2 spectra 35 / 37 (a whole pair), 3 spectra 49 / 45, 4
+// spectra 51 / 51, 12 taps 2 spectra 43 / 40; 2^20 single-pol 8 taps 1 spectrum
+// 97 / 78, 2 spectra 114 / 103, 3 spectra 131 / 124, 4 spectra 133 / 143, 6 taps 1
 // spectrum 81 / 74, 2 spectra 93 / 98; dual-pol 16 taps 1 spectrum 130 / 113, 2
-// spectra 139 / 177.
-static int short_calls(const vspec_plan *p) {
+// spectra 139 / 177. Bit n: calls of n spectra.
+static unsigned short_calls(const vspec_plan *p) {
     if (p->fused || p->mode != VSPEC_PFB || p->req_n2 || p->req_cols ||
         (p->flags & (VSPEC_PLAN_TENSOR | VSPEC_PLAN_KAHAN | VSPEC_PLAN_TENSOR_INT8 | VSPEC_PLAN_RING)))
         return 0;
-    if (p->N == 1 << 19) return p->npol == 1 || p->P > 8 ? 4 : 0;
+    constexpr unsigned one = 1u << 1, two = 1u << 2, three = 1u << 3;
+    if (p->N == 1 << 19) return p->P > 8 ? one | two | three : p->npol == 1 ? one | three : 0;
     if (p->N != 1 << 20) return 0;
-    if (p->npol == 2) return p->P > 8 ? 2 : 0;
-    return p->P > 8 || p->P < 6 ? 0 : p->P == 6 ? 2 : 4;  // (more than 8 taps: the gather form itself)
+    if (p->npol == 2) return p->P > 8 ? one : 0;
+    return p->P > 8 || p->P < 6 ? 0 : p->P == 6 ? one : one | two | three;  // (more than 8 taps: the gather form itself)
 }
 static vspec_status setup_short(vspec_plan *p) {
-    const int below = short_calls(p);
-    if (!below) return VSPEC_OK;
+    const unsigned counts = short_calls(p);
+    if (!counts) return VSPEC_OK;
     vspec_plan *q = new (std::nothrow) vspec_plan();
     if (!q) return VSPEC_ERR_OOM;
     q->N = p->N;
@@ -1377,14 +1380,14 @@ static vspec_status setup_short(vspec_plan *p) {
     q->window = p->window;
     q->flags = p->flags;
     q->owner = p;
-    q->short_cap = below - 1;
+    q->short_cap = ilog2((int)counts);
     const vspec_status st = build_plan(q);
     if (st != VSPEC_OK) {
         free_plan(q);
         return st == VSPEC_ERR_OOM ? VSPEC_OK : st;  // without it every call runs the plan's own kernels
     }
     p->short_plan = q;
-    p->short_below = below;
+    p->short_counts = counts;
     p->scratch_bytes += q->scratch_bytes;
     return VSPEC_OK;
 }
@@ -1541,8 +1544,12 @@ vspec_status vspec_plan_describe(const vspec_plan *plan, char *buf, size_t len) 
         if (plan->row_plan) d += " | " + two_kernel(plan->row_plan);
     } else {
         d = two_kernel(plan);
-        if (plan->short_plan)
-            d += " | below " + std::to_string(plan->short_below) + " spectra " + two_kernel(plan->short_plan);
+        if (plan->short_plan) {
+            d += " | spectra";
+            for (int n = 1; n < 32; n++)
+                if (plan->short_counts >> n & 1) d += (d.back() == 'a' ? "=" : ",") + std::to_string(n);
+            d += " " + two_kernel(plan->short_plan);
+        }
     }
     const size_t n = std::min(len - 1, d.size());
     std::memcpy(buf, d.data(), n);
@@ -2223,7 +2230,7 @@ static vspec_status execute_one(vspec_plan *p, const int8_t *d_in, int nspectra,
                                 cudaStream_t st) {
     if (p->ring) return run_ring(p, d_in, nspectra, d_accum, st);
     // (a plan tuned to its own launch shape keeps it)
-    if (nspectra < p->short_below && p->blocks_a == 0 && p->blocks_b == 0 && nspectra <= p->sc_max)
+    if (nspectra < 32 && (p->short_counts >> nspectra & 1) && p->blocks_a == 0 && p->blocks_b == 0 && nspectra <= p->sc_max)
         return run_two_kernel(p->short_plan, d_in, nspectra, d_accum, st, nullptr);
     if (!p->fused) return run_two_kernel(p, d_in, nspectra, d_accum, st, nullptr);
     if (p->row_plan) return run_two_kernel(p->row_plan, d_in, nspectra, d_accum, st, nullptr);
