@@ -194,7 +194,8 @@ struct vspec_plan {
     vspec_plan *row_plan = nullptr;
     // long transforms: calls of n spectra, bit n of short_counts set, run this
     // plan, the general or tap-gather kernel A (setup_short). Its own short_cap,
-    // if set, is its longest call; its coefficients are the owner's.
+    // if set, is its longest call; its coefficients, chunk scratch and partial
+    // sums are the owner's (these two at the time of a call).
     vspec_plan *short_plan = nullptr;
     unsigned short_counts = 0;
     int short_cap = 0;
@@ -589,7 +590,8 @@ void free_plan(vspec_plan *p) {
     if (p->short_plan) free_plan(p->short_plan);
     for (cudaEvent_t e : p->event_pool) cudaEventDestroy(e);
     release_host_pipeline(p);
-    if (!p->short_cap) cudaFree(p->coef);
+    if (p->short_cap) p->coef = nullptr, p->Z = p->partial = nullptr;  // the owner's
+    cudaFree(p->coef);
     cudaFree(p->twA);
     cudaFree(p->twB);
     cudaFree(p->twZ);
@@ -1191,8 +1193,10 @@ vspec_status build_plan(vspec_plan *p) {
         if ((st = dev_alloc((void **)&p->ring_ctl, sizeof(int) * (2 + 2 * (size_t)kRingSlotsPerLaunch), &tot)))
             return st;
     }
-    if ((st = dev_alloc(&p->Z, z_bytes(p, std::max(1, p->sc_alloc)), &tot))) return st;
-    if ((st = dev_alloc(&p->partial, (size_t)p->slots_cap * N * accel, &tot))) return st;
+    if (!p->short_cap) {
+        if ((st = dev_alloc(&p->Z, z_bytes(p, std::max(1, p->sc_alloc)), &tot))) return st;
+        if ((st = dev_alloc(&p->partial, (size_t)p->slots_cap * N * accel, &tot))) return st;
+    }
     if (p->tc || p->tc_cols || p->ring) {
         if ((st = dev_alloc((void **)&p->tc_status, sizeof(int), &tot))) return st;
         VSPEC_CUDA(cudaMemset(p->tc_status, 0, sizeof(int)));
@@ -1382,7 +1386,7 @@ static vspec_status setup_short(vspec_plan *p) {
     q->owner = p;
     q->short_cap = ilog2((int)counts);
     const vspec_status st = build_plan(q);
-    if (st != VSPEC_OK) {
+    if (st != VSPEC_OK || q->slots_cap > p->slots_cap || q->sc_max > p->sc_alloc) {
         free_plan(q);
         return st == VSPEC_ERR_OOM ? VSPEC_OK : st;  // without it every call runs the plan's own kernels
     }
@@ -2230,8 +2234,12 @@ static vspec_status execute_one(vspec_plan *p, const int8_t *d_in, int nspectra,
                                 cudaStream_t st) {
     if (p->ring) return run_ring(p, d_in, nspectra, d_accum, st);
     // (a plan tuned to its own launch shape keeps it)
-    if (nspectra < 32 && (p->short_counts >> nspectra & 1) && p->blocks_a == 0 && p->blocks_b == 0 && nspectra <= p->sc_max)
+    if (nspectra < 32 && (p->short_counts >> nspectra & 1) && p->blocks_a == 0 && p->blocks_b == 0 &&
+        nspectra <= p->sc_max) {
+        p->short_plan->Z = p->Z;
+        p->short_plan->partial = p->partial;
         return run_two_kernel(p->short_plan, d_in, nspectra, d_accum, st, nullptr);
+    }
     if (!p->fused) return run_two_kernel(p, d_in, nspectra, d_accum, st, nullptr);
     if (p->row_plan) return run_two_kernel(p->row_plan, d_in, nspectra, d_accum, st, nullptr);
     if (p->assist && nspectra >= p->two_kernel_from)

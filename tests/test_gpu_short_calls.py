@@ -1,7 +1,8 @@
 """Calls of one to a few spectra of the longest pre-filters, on either side of
 the length below which they take the tap-gather kernel: every count gives the
 oracle's spectrum, the two paths' calls add up in one accumulator, a tuned plan
-keeps its own kernels, and a captured call replays."""
+keeps its own kernels, a captured call replays, and a scratch that was replaced is
+the one that the next call uses."""
 import numpy as np
 import pytest
 
@@ -58,3 +59,11 @@ def test_short_calls_match_oracle_and_add_up(oracle_mod, n, p, npol, counts):
         plan.dump(acc)
         plan.execute(d_in, 1, acc)
         assert_close(spectrum().reshape(o.shape), o, what="tuned")
+        for chunk in (2, 8):  # the scratch that both plans use, smaller and larger than before
+            plan.tune(blocks_a=0, chunk_spectra=chunk)
+            plan.trim_scratch()
+            for count in (1, 3):
+                plan.dump(acc)
+                plan.execute(d_in, count, acc)
+                o = oracle(0, count)
+                assert_close(spectrum().reshape(o.shape), o, what=f"{count} spectra, chunks of {chunk}")
